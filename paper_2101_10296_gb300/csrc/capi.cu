@@ -30,6 +30,7 @@ void free_work(DevWork &w) {
     cudaFree(w.slot_cone);
     cudaFree(w.warp_graph);
     cudaFree(w.rec_hi);
+    cudaFree(w.rec_cnt);
     cudaFree(w.rec_wk);
     cudaFree(w.rec_cw);
     w = DevWork{};
@@ -68,18 +69,23 @@ uint64_t host_shell_block(const DevCone &C, const std::vector<uint64_t> &tab, ui
     return m;
 }
 
-// Builds the slot list for R register qubits over the given plan indices:
-// cones sorted by (G_c = 2^max(n_in - R, 0) descending, graph, plan order)
+// The slot list for R register qubits over the given plan indices: order (plan
+// indices in list order), the first slot and the slot count of each, and the
+// number of slots.
+struct SlotList {
+    std::vector<int32_t> order;
+    std::vector<int64_t> start, count;
+    int64_t slots = 0;
+};
+
+// Cones sorted by (G_c = 2^max(n_in - R, 0) descending, graph, plan order)
 // and packed back to back, T_c slots each (a multiple of G_c, so every cone
 // starts at a multiple of its own G_c and its lane-qubit groups never
-// straddle a cone boundary); a new graph starts on a fresh warp.  Then the
-// slot records (see RegWork): for slot s of cone c at offset t = s - start_c
-// the thread holds inner qubits R..n_in-1 in the low bits of t and block
-// group t >> max(n_in - R, 0); register bits [2, nr) are inner qubits (nr =
-// min(n_in, R)) and bits [nr, R) pick one of 2^(R - nr) blocks of the group.
-int build_work(const std::vector<DevCone> &hc, const std::vector<uint64_t> &shell_tab,
-               const std::vector<int32_t> &idx, int R, bool wide, DevWork &w) {
-    std::vector<int32_t> order(idx);
+// straddle a cone boundary); a new graph starts on a fresh warp.
+SlotList slot_list(const std::vector<DevCone> &hc, const std::vector<int32_t> &idx, int R) {
+    SlotList list;
+    std::vector<int32_t> &order = list.order;
+    order = idx;
     auto G = [&](int32_t i) { return int64_t(1) << std::max(hc[i].n_in - R, 0); };
     auto T = [&](int32_t i) {
         const int sb = std::max(R - hc[i].n_in, 0);
@@ -89,16 +95,30 @@ int build_work(const std::vector<DevCone> &hc, const std::vector<uint64_t> &shel
         if (G(a) != G(b)) return G(a) > G(b);
         return hc[a].graph < hc[b].graph;
     });
-    std::vector<int64_t> start(order.size() + 1, 0);
+    list.start.assign(order.size(), 0);
+    list.count.assign(order.size(), 0);
     int64_t pos = 0;
     for (size_t i = 0; i < order.size(); ++i) {
         if (i > 0 && hc[order[i]].graph != hc[order[i - 1]].graph) pos = (pos + 31) / 32 * 32;
-        start[i] = pos;
-        pos += T(order[i]);
+        list.start[i] = pos;
+        list.count[i] = T(order[i]);
+        pos += list.count[i];
     }
-    pos = (pos + 31) / 32 * 32;
-    start[order.size()] = pos;
-    const int64_t slots = pos;
+    list.slots = (pos + 31) / 32 * 32;
+    return list;
+}
+
+// Work list of the general kernel: the slot list and its records (see
+// RegWork): for slot s of cone c at offset t = s - start_c the thread holds
+// inner qubits R..n_in-1 in the low bits of t and block group t >> max(n_in -
+// R, 0); register bits [2, nr) are inner qubits (nr = min(n_in, R)) and bits
+// [nr, R) pick one of 2^(R - nr) blocks of the group.
+int build_work(const std::vector<DevCone> &hc, const std::vector<uint64_t> &shell_tab,
+               const std::vector<int32_t> &idx, int R, bool wide, DevWork &w) {
+    const SlotList list = slot_list(hc, idx, R);
+    const std::vector<int32_t> &order = list.order;
+    const std::vector<int64_t> &start = list.start;
+    const int64_t slots = list.slots;
     const int64_t warps = slots / 32;
     w.slots = slots;
     w.warps = warps;
@@ -114,7 +134,7 @@ int build_work(const std::vector<DevCone> &hc, const std::vector<uint64_t> &shel
         // the cone owning the slot: the last one starting at or before it
         while (ci + 1 < order.size() && start[ci + 1] <= sl) ++ci;
         const DevCone &C = hc[size_t(order[ci])];
-        const bool active = sl < start[ci] + T(order[ci]);
+        const bool active = sl < start[ci] + list.count[ci];
         scone[size_t(sl)] = order[ci] | (active ? 0 : int32_t(0x80000000u));
         if (sl % 32 == 0) wgraph[size_t(sl / 32)] = C.graph;
         const int64_t t = active ? sl - start[ci] : 0;  // padding: the cone's first slot, weight 0
@@ -164,6 +184,48 @@ int build_work(const std::vector<DevCone> &hc, const std::vector<uint64_t> &shel
     if (e == cudaSuccess)
         e = cudaMemcpy(w.warp_graph, wgraph.data(), wgraph.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy");
+    return QAOA_OK;
+}
+
+// Work list of the depth-2 kernel: the slot list from the host, the records
+// filled on the device from the uploaded cones and shell table.
+int build_depth2_work(const std::vector<DevCone> &hc, const std::vector<int32_t> &idx, int R,
+                      const qaoa_device_plan *d, DevWork &w) {
+    const SlotList list = slot_list(hc, idx, R);
+    w.slots = list.slots;
+    w.warps = list.slots / 32;
+    w.n = int32_t(list.order.size());
+    if (list.order.empty()) return QAOA_OK;
+    std::vector<int32_t> wgraph(size_t(w.warps), 0), scone(size_t(w.slots), 0);
+    std::vector<int64_t> cone_start(hc.size(), 0);
+    for (size_t i = 0; i < list.order.size(); ++i) {
+        const int32_t c = list.order[i];
+        const int64_t first = list.start[i], last = first + list.count[i];
+        const int64_t next = i + 1 < list.order.size() ? list.start[i + 1] : list.slots;
+        cone_start[size_t(c)] = first;
+        std::fill(scone.begin() + first, scone.begin() + last, c);
+        std::fill(scone.begin() + last, scone.begin() + next, c | int32_t(0x80000000u));  // padding
+        for (int64_t v = (first + 31) / 32; v * 32 < next; ++v) wgraph[size_t(v)] = hc[size_t(c)].graph;
+    }
+    const size_t n_rec = size_t(w.slots) << (R - 2);
+    int64_t *start = nullptr;
+    cudaError_t e;
+    if ((e = cudaMalloc(&w.slot_cone, scone.size() * sizeof(int32_t))) != cudaSuccess ||
+        (e = cudaMalloc(&w.warp_graph, wgraph.size() * sizeof(int32_t))) != cudaSuccess ||
+        (e = cudaMalloc(&w.rec_cnt, 2 * n_rec * sizeof(uint32_t))) != cudaSuccess ||
+        (e = cudaMalloc(&w.rec_wk, n_rec * sizeof(float))) != cudaSuccess ||
+        (e = cudaMalloc(&start, cone_start.size() * sizeof(int64_t))) != cudaSuccess)
+        return cuda_fail(e, "cudaMalloc");
+    e = cudaMemcpy(w.slot_cone, scone.data(), scone.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(w.warp_graph, wgraph.data(), wgraph.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(start, cone_start.data(), cone_start.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = build_depth2_records(d->cones, d->shell, w.slot_cone, start, w.slots, R, d->cmax1, w.rec_cnt, w.rec_wk);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // start is read by the kernel
+    cudaFree(start);
+    if (e != cudaSuccess) return cuda_fail(e, "work list upload");
     return QAOA_OK;
 }
 
@@ -269,7 +331,7 @@ int ensure_uploaded(const qaoa_plan *plan) {
 // points per warp task, gives at least four waves of 8 warps per SM.
 int reg_bits_for(const qaoa_device_plan *d, int64_t n_points) {
     if (d->reg_bits_grad == 4 || d->reg_bits_grad == 5) return d->reg_bits_grad;
-    const int64_t tasks = d->reg_g[1].warps * ((n_points + 31) / 32);
+    const int64_t tasks = d->reg[1].warps * ((n_points + 31) / 32);
     return tasks >= int64_t(sm_count()) * 8 * 4 ? 5 : 4;
 }
 
@@ -279,6 +341,53 @@ int64_t tuned_grid(const qaoa_device_plan *d, int occupancy_grid) {
     if (d->blocks_per_sm <= 0) return occupancy_grid;
     return std::min<int64_t>(occupancy_grid, int64_t(sm_count()) * d->blocks_per_sm);
 }
+
+}  // namespace
+
+namespace qaoa {
+// Points per warp task: up to 32, in the depth-2 kernel as many as leave room
+// for the resident blocks its registers allow, in the general one phase tables
+// of at most 8 KB per warp; halved while the tasks would not give every SM 16
+// warps (small plans: more tasks of fewer points).  A tuned value is held to
+// what a block may use.
+cudaError_t launch_reg(const qaoa_device_plan *d, RegLaunch &L, bool grad, int rg, int points_per_task,
+                       cudaStream_t s) {
+    const int p = L.p;
+    int64_t fit, cap;
+    if (d->depth2) {
+        const int64_t point = int64_t(depth2_point_bytes(L.cmax1));
+        const int64_t fixed = int64_t(depth2_smem_bytes(0, L.cmax1, grad));
+        const int blocks = depth2_blocks(grad, rg);
+        cap = (kRegMaxSmem - fixed) / (kRegBlock / 32) / point;
+        fit = std::min<int64_t>(cap, (smem_per_block(blocks) - fixed) / (kRegBlock / 32) / point);
+    } else {
+        const int64_t row = int64_t(p) * ((L.cmax1 + 1) * int64_t(sizeof(float2)) + kRegKpow * int64_t(sizeof(float)));
+        fit = 8192 / row;
+        cap = 12288 / row;
+    }
+    int64_t jpt = points_per_task;
+    if (jpt <= 0) {
+        jpt = std::min<int64_t>(32, std::max<int64_t>(1, fit));
+        while (jpt > 1 && L.work.warps * ((L.n_points + jpt - 1) / jpt) < int64_t(sm_count()) * 16) jpt = (jpt + 1) / 2;
+    }
+    jpt = std::min<int64_t>(jpt, std::max<int64_t>(1, cap));
+    L.jpt = int32_t(std::min<int64_t>(jpt, L.n_points));
+    const int64_t tasks = L.work.warps * ((L.n_points + L.jpt - 1) / L.jpt);
+    const bool wide = L.cmax1 - 1 > 32;
+    int occ;
+    if (d->depth2)
+        occ = depth2_grid(grad, rg, L.cmax1, depth2_smem_bytes(L.jpt, L.cmax1, grad));
+    else if (grad)
+        occ = reg_grad_grid(wide, reg_smem_bytes(L.jpt, p, L.cmax1, true), p, rg);
+    else
+        occ = reg_energy_grid(wide, reg_smem_bytes(L.jpt, p, L.cmax1, false));
+    const int grid = int(std::max<int64_t>(1, std::min<int64_t>(tuned_grid(d, occ), (tasks + 3) / 4)));
+    if (d->depth2) return launch_depth2(L, grad, rg, grid, s);
+    return grad ? launch_reg_grad(L, wide, rg, grid, s) : launch_reg_energy(L, wide, grid, s);
+}
+}  // namespace qaoa
+
+namespace {
 
 // Large-state cones: per shape, waves of blocks that fit the scratch budget,
 // each wave streamed through the shape's pass list.
@@ -384,7 +493,6 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
         cudaFreeAsync(lut, s);
         return cuda_fail(e, "cudaMallocAsync");
     }
-    const bool wide = d->cmax1 - 1 > 32;
     PrepArgs pa;
     pa.params = params;
     pa.G = G;
@@ -453,25 +561,6 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
         RegLaunch L;
         L.n_points = n_points;
         L.p = p;
-        // points per warp task: up to 32, phase tables of at most 8 KB per warp,
-        // halved while the tasks would not give every SM 16 warps (small
-        // plans: more tasks of fewer points); a tuned value is held to the
-        // 48 KB of shared memory of 4 warps
-        {
-            // one point's phase tables, mixer data and kappa powers
-            const int64_t row_bytes = int64_t(p) * ((d->cmax1 + 1) * int64_t(sizeof(float2)) + kRegKpow * int64_t(sizeof(float)));
-            const int rgi = reg_bits_for(d, n_points) - 4;
-            const int64_t warps = grad ? d->reg_g[rgi].warps : d->reg_e.warps;
-            int64_t jpt = d->points_per_task;
-            if (jpt <= 0) {
-                jpt = std::min<int64_t>(32, std::max<int64_t>(1, 8192 / row_bytes));
-                while (jpt > 1 && warps * ((n_points + jpt - 1) / jpt) < int64_t(sm_count()) * 16) jpt = (jpt + 1) / 2;
-            }
-            jpt = std::min<int64_t>(jpt, std::max<int64_t>(1, 12288 / row_bytes));
-            L.jpt = int32_t(std::min<int64_t>(jpt, n_points));
-        }
-        const size_t smem = reg_smem_bytes(L.jpt, p, d->cmax1, grad != nullptr);
-        const int64_t tasks_per = (n_points + L.jpt - 1) / L.jpt;
         L.cmax1 = d->cmax1;
         L.lut = lut;
         L.mix = mix;
@@ -481,21 +570,10 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
         L.terms = terms;
         L.status = d->status;
         L.norm = norm && !grad ? 1 : 0;
-        if (grad) {
-            const int rg = reg_bits_for(d, n_points);
-            L.work = as_reg(d, d->reg_g[rg - 4]);
-            if (L.work.warps > 0) {
-                int64_t grid = std::min<int64_t>(tuned_grid(d, reg_grad_grid(wide, smem, p, rg)),
-                                                 (L.work.warps * tasks_per + 3) / 4);
-                e = launch_reg_grad(L, wide, rg, int(std::max<int64_t>(grid, 1)), s);
-            }
-        } else {
-            L.work = as_reg(d, d->reg_e);
-            if (L.work.warps > 0) {
-                int64_t grid = std::min<int64_t>(tuned_grid(d, reg_energy_grid(wide, smem)), (L.work.warps * tasks_per + 3) / 4);
-                e = launch_reg_energy(L, wide, int(std::max<int64_t>(grid, 1)), s);
-            }
-        }
+        const bool g = grad != nullptr;
+        const int rg = g ? reg_bits_for(d, n_points) : kRegBitsEnergy;
+        L.work = as_reg(d, d->reg[rg - 4]);
+        if (L.work.warps > 0) e = launch_reg(d, L, g, rg, d->points_per_task, s);
         if (L.work.warps > 0) dm->all_launches += 1;
         if (e == cudaSuccess && !d->big.empty()) e = run_big(d, plan, n_points, params, lut, mix, kpow, energy, grad, terms, norm, s);
     }
@@ -519,9 +597,8 @@ extern "C" void qaoa_device_release(qaoa_plan *plan) {
     cudaGetDevice(&cur);
     if (d->device >= 0) cudaSetDevice(d->device);
     cudaFree(d->cones);
-    free_work(d->reg_e);
-    free_work(d->reg_g[0]);
-    free_work(d->reg_g[1]);
+    free_work(d->reg[0]);
+    free_work(d->reg[1]);
     free_work(d->reg_p1);
     for (auto &bs : d->big) {
         cudaFree(bs.d_cones);
@@ -682,9 +759,13 @@ extern "C" int qaoa_plan_upload(qaoa_plan *plan) {
             cudaMemcpy(d->shell, shell_tab.data(), shell_tab.size() * sizeof(uint64_t), cudaMemcpyHostToDevice);
     }
     const bool wide = cmax > 32;  // the kernels' cut-word width (as at launch)
-    if (rc == QAOA_OK) rc = build_work(hc, shell_tab, reg_idx, kRegBitsEnergy, wide, d->reg_e);
-    if (rc == QAOA_OK) rc = build_work(hc, shell_tab, reg_idx, 4, wide, d->reg_g[0]);
-    if (rc == QAOA_OK) rc = build_work(hc, shell_tab, reg_idx, 5, wide, d->reg_g[1]);
+    // the depth-2 kernel's lists at p = 2 when every register cone's last layer
+    // mixes the edge alone (always, without QAOA_FULL_CONE)
+    d->depth2 = plan->p == 2;
+    for (int32_t i : reg_idx) d->depth2 = d->depth2 && hc[size_t(i)].k[1] == 2;
+    for (int rb = 4; rb <= 5 && rc == QAOA_OK; ++rb)
+        rc = d->depth2 ? build_depth2_work(hc, reg_idx, rb, d, d->reg[rb - 4])
+                       : build_work(hc, shell_tab, reg_idx, rb, wide, d->reg[rb - 4]);
     // depth 1 with every register cone mixing qubits 0 and 1 only (its inner
     // part): the depth-1 kernel's list
     bool p1 = plan->p == 1 && !reg_idx.empty();

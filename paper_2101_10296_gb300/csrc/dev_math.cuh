@@ -8,6 +8,12 @@ namespace qaoa {
 
 constexpr unsigned kFull = 0xffffffffu;
 
+// The warp's index in its block, broadcast from lane 0 so that the compiler
+// knows it is the same in every lane: branches and loop bounds that follow from
+// it are then warp-uniform.  Where it cannot tell, it surrounds every shuffle
+// inside with a reconvergence path of about seven instructions.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(kFull, int(threadIdx.x >> 5), 0); }
+
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }

@@ -86,11 +86,17 @@ __device__ __forceinline__ uint64_t shell_block(const DevCone *__restrict__ C, c
 // and register bits 2.. -- and rec_wk[k * slots + s] the multiplicity of the
 // block index i belongs to (0 past the cone's blocks and in padding slots).
 // Words are uint32 when every cone has at most 32 cut bits, else uint64.
+//
+// The lists of the depth-2 kernel hold rec_cnt instead of rec_hi: the cut values
+// themselves, of amplitudes 4k .. 4k + 3 in rec_cnt[k * slots + s], one byte
+// each, scaled by 4 when every cone has at most 31 cut bits, else by 2; then
+// the same after the first layer's flips (from row S = 2^(R-2) on).
 struct RegWork {
     const DevCone *cones = nullptr;       // plan order
     const int32_t *slot_cone = nullptr;   // plan index of each slot's cone; bit 31: padding slot
     const int32_t *warp_graph = nullptr;  // the graph of each warp's slots
     const void *rec_hi = nullptr;         // slot records (above)
+    const uint32_t *rec_cnt = nullptr;
     const float *rec_wk = nullptr;
     const uint2 *rec_cw = nullptr;        // depth-1 work lists: per block the four cut values and the multiplicity
     int32_t n_cones = 0;
@@ -233,5 +239,34 @@ inline size_t reg_smem_bytes(int jpt, int p, int cmax1, bool grad) {
             (size_t(jpt) * p * kRegKpow + size_t(reg_outputs(p, grad)) * reg_group(p, grad) * 32 +
              size_t(reg_lane_words(p)) * 32) * sizeof(float));
 }
+
+// Depth-2 kernel (depth2_kernel.cuh; plans of depth 2 whose register cones are
+// all pruned): bytes of one layer's phase-table row in shared memory (narrow:
+// at most 31 cut bits, 32 entries), floats of a point's parameters, and a
+// block's dynamic shared memory.
+// Resident 128-thread blocks per SM: 128 registers for the energy and the
+// adjoint with four register qubits, 255 with five (energy at 3 and 5 blocks:
+// 752 and 842 against 734 us on four random cubic graphs of 2,000 vertices and
+// 64 points; the adjoint with four at 3 and 5: 2858 and 2909 against 2677 us).
+__host__ __device__ constexpr int depth2_blocks(bool grad, int rg) { return grad && rg == 5 ? 2 : 4; }
+constexpr int kDepth2WideRow = 544;  // 2 x 68 entries, a multiple of 32 bytes
+constexpr int kDepth2Params = 4 + kRegKpow;
+__host__ __device__ constexpr bool depth2_narrow(int cmax1) { return cmax1 <= 32; }
+__host__ __device__ constexpr int depth2_row_bytes(bool narrow) { return narrow ? 256 : kDepth2WideRow; }
+inline size_t depth2_point_bytes(int cmax1) {
+    return 2 * size_t(depth2_row_bytes(depth2_narrow(cmax1))) + kDepth2Params * sizeof(float);
+}
+inline size_t depth2_smem_bytes(int jpt, int cmax1, bool grad) {
+    return size_t(kRegBlock / 32) * (size_t(jpt) * depth2_point_bytes(cmax1) +
+                                     size_t(reg_outputs(2, grad)) * reg_group(2, grad) * 32 * sizeof(float));
+}
+// rg: register qubits per thread of the adjoint (4 or 5)
+int depth2_grid(bool grad, int rg, int cmax1, size_t smem);
+cudaError_t launch_depth2(const RegLaunch &a, bool grad, int rg, int grid, cudaStream_t s);
+cudaError_t depth2_prepare();
+// Fills the records of a depth-2 work list on the device (legacy default
+// stream); start: device int64 per cone, its first slot.
+cudaError_t build_depth2_records(const DevCone *cones, const uint64_t *shell, const int32_t *slot_cone,
+                                 const int64_t *start, int64_t slots, int R, int cmax1, uint32_t *cnt, float *wk);
 
 }  // namespace qaoa

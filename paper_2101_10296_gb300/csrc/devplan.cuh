@@ -12,6 +12,7 @@ struct DevWork {
     int32_t *slot_cone = nullptr;   // plan index of every slot's cone; bit 31 set in padding slots
     int32_t *warp_graph = nullptr;  // graph of every warp's slots
     void *rec_hi = nullptr;         // [S][slots] cut words (uint32 or uint64, see RegWork)
+    uint32_t *rec_cnt = nullptr;    // depth-2 lists: [2][S][slots] cut values, one byte per amplitude
     float *rec_wk = nullptr;        // [S][slots] block multiplicities
     uint2 *rec_cw = nullptr;        // depth-1 lists: [kP1Blocks][slots] cut values and multiplicity
     int64_t slots = 0, warps = 0;
@@ -35,8 +36,11 @@ struct qaoa_device_plan {
     int device = -1;
     qaoa::DevCone *cones = nullptr;
     int64_t n_cones = 0;
-    DevWork reg_e;       // work list of the energy kernels
-    DevWork reg_g[2];    // of the adjoint kernels with 4 and 5 register qubits
+    // Work lists with 4 and 5 register qubits per thread: the energy takes 5, the
+    // adjoint either.  depth2: they are those of the depth-2 kernel (p = 2 and
+    // every register cone's last layer mixes the edge alone)
+    DevWork reg[2];
+    bool depth2 = false;
     DevWork reg_p1;      // of the depth-1 kernel (p = 1 plans whose register cones all mix qubits 0, 1 only)
     std::vector<BigShape> big;
     size_t big_budget = size_t(1) << 30;  // scratch bytes per call for big cones
@@ -54,6 +58,12 @@ struct qaoa_device_plan {
     int64_t all_launches = 0;
 };
 
+namespace qaoa {
+// Launches the register-resident cones of L.work (capi.cu) on the depth-2 or
+// the general kernel; points_per_task 0: the default.  Fills L.jpt.
+cudaError_t launch_reg(const qaoa_device_plan *d, RegLaunch &L, bool grad, int rg, int points_per_task, cudaStream_t s);
+}  // namespace qaoa
+
 // The register kernels' view of a work list.
 inline qaoa::RegWork reg_work(const qaoa_device_plan *d, const DevWork &w) {
     qaoa::RegWork r;
@@ -61,6 +71,7 @@ inline qaoa::RegWork reg_work(const qaoa_device_plan *d, const DevWork &w) {
     r.slot_cone = w.slot_cone;
     r.warp_graph = w.warp_graph;
     r.rec_hi = w.rec_hi;
+    r.rec_cnt = w.rec_cnt;
     r.rec_wk = w.rec_wk;
     r.rec_cw = w.rec_cw;
     r.n_cones = w.n;

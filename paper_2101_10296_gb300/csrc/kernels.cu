@@ -194,6 +194,7 @@ cudaError_t reg_prepare() {
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, kRegMaxSmem);
     if (e == cudaSuccess) e = reg_grad_prepare();
     if (e == cudaSuccess) e = reg_p1_prepare();
+    if (e == cudaSuccess) e = depth2_prepare();
     if (e == cudaSuccess) done.insert(dev);
     return e;
 }

@@ -158,13 +158,11 @@ extern "C" int qaoa_energy_noalloc(const qaoa_plan *plan, int64_t n_points, cons
         const int64_t tasks = L.work.warps * ((n_points + L.jpt - 1) / L.jpt);
         const int64_t grid = std::min<int64_t>(reg_p1_grid(false, smem), (tasks + 3) / 4);
         e = launch_reg_p1(L, false, int(std::max<int64_t>(grid, 1)), s);
-    } else if (e == cudaSuccess && d->reg_e.warps > 0) {
+    } else if (e == cudaSuccess && d->reg[kRegBitsEnergy - 4].warps > 0) {
         RegLaunch L;
-        L.work = reg_work(d, d->reg_e);
+        L.work = reg_work(d, d->reg[kRegBitsEnergy - 4]);
         L.n_points = n_points;
         L.p = p;
-        const int64_t row_bytes = int64_t(p) * ((d->cmax1 + 1) * int64_t(sizeof(float2)) + kRegKpow * int64_t(sizeof(float)));
-        L.jpt = int32_t(std::min<int64_t>(std::min<int64_t>(8, std::max<int64_t>(1, 6144 / row_bytes)), n_points));
         L.cmax1 = d->cmax1;
         L.lut = lut;
         L.mix = mix;
@@ -173,11 +171,7 @@ extern "C" int qaoa_energy_noalloc(const qaoa_plan *plan, int64_t n_points, cons
         L.grad = nullptr;
         L.terms = terms_dev;
         L.status = d->status;
-        const bool wide = d->cmax1 - 1 > 32;
-        const size_t smem = reg_smem_bytes(L.jpt, p, d->cmax1, false);
-        const int64_t tasks = d->reg_e.warps * ((n_points + L.jpt - 1) / L.jpt);
-        const int64_t grid = std::min<int64_t>(reg_energy_grid(wide, smem), (tasks + 3) / 4);
-        e = launch_reg_energy(L, wide, int(std::max<int64_t>(grid, 1)), s);
+        e = launch_reg(d, L, false, kRegBitsEnergy, 0, s);
     }
     // large-state cones: waves sized to the room left in the array
     if (e == cudaSuccess && !d->big.empty()) {

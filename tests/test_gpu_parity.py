@@ -959,6 +959,40 @@ def test_adjoint_register_widths_match_oracle(q, graph, p, signs):
     assert plan.device_status() == 0
 
 
+@pytest.mark.parametrize("P", [1, 33])
+@pytest.mark.parametrize("graph,weight", [
+    ((2, np.array([[0, 1]])), 1), (I.path(5), 1), (I.star(5), 1), (I.complete(4), 1), (I.cycle(11), 3),
+    (I.random_regular(10, 3, 2), 1), (I.random_regular(12, 4, 1), 1), (I.complete(6), 2), (I.complete(7), 3),
+    (I.random_regular(12, 3, 4), -2)],
+    ids=["edge", "path", "star", "K4", "cycle-w3", "cubic", "4-regular", "K6-w2", "K7-w3", "cubic-w-2"])
+def test_depth2_kernel_edges(q, graph, weight, P):
+    """p = 2 register cones from two to nine inner qubits (fewer than a thread holds, and up to four on
+    the lanes), narrow and wide count bytes (31 and more cut bits), one point and a partial task: terms,
+    energies and both adjoint widths against the FP64 oracle."""
+    n, edges = graph
+    w = np.full(len(edges), weight)
+    th = I.draw_params(2, P, 11)
+    plan = q.Plan(graph, 2, weights=[w], orbits=False)
+    e, terms = plan.energy(_params(th), terms=True)
+    pick = [0] if P == 1 else [0, P - 1]
+    for j in pick:
+        ref = [O.lightcone_term(n, edges, ed, th[j], 2, weights=w) for ed in edges]
+        assert np.abs(terms.cpu().numpy()[:, j] - ref).max() <= 1e-5
+        eref = float((w * (1 - np.array(ref)) / 2).sum())
+        gref = O.grad_adjoint(n, edges, th[j], 2, weights=w)
+        gref = gref[1] if isinstance(gref, tuple) else gref
+        assert abs(e.cpu().numpy()[0, j] - eref) <= 1e-6 * np.abs(w).sum()
+        for bits in (4, 5):
+            plan.set_tuning(reg_bits_grad=bits)
+            eg, g = plan.energy_grad(_params(th))
+            assert abs(eg.cpu().numpy()[0, j] - eref) <= 1e-6 * np.abs(w).sum()
+            _check_grad(g.cpu().numpy()[0, j], gref, energy=np.abs(w).sum())
+    norms = plan.norms(_params(th)).cpu().numpy()
+    assert np.abs(norms - 1).max() <= 1e-5
+    assert plan.device_status() == 0
+
+
+
 def test_tuning_leaves_results_unchanged(q):
     plan, G = _mixed_plan(q)
     th = _params(np.stack([I.draw_params(3, 7, 30 + g) for g in range(G)]))
