@@ -22,7 +22,7 @@ constexpr int NR = 1 << kBigRegBits;
 template <bool GRAD>
 __global__ void __launch_bounds__(128) big_pass_kernel(const __grid_constant__ BigLaunch L) {
     const int lane = threadIdx.x & 31;
-    const int64_t gw = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp_index();
     const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
     const BigPass &ps = L.pass;
     const int b = ps.b;
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(128) big_pass_kernel(const __grid_constant__ B
 // No cut words or tables, so far fewer registers and more loads in flight.
 __global__ void __launch_bounds__(128, 4) big_mix_kernel(const __grid_constant__ BigLaunch L) {
     const int lane = threadIdx.x & 31;
-    const int64_t gw = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp_index();
     const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
     const BigPass &ps = L.pass;
     const int b = ps.b;

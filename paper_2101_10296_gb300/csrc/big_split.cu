@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(128, GRAD ? QAOA_SPLIT_GRAD_BLOCKS : 3) split_
     constexpr int T = RB + 5;
     constexpr int NW = NR / 4;  // packed cut counts, 4 registers per word
     const int lane = threadIdx.x & 31;
-    const int64_t gw = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp_index();
     const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
     const int nin = L.n_in;
     const int p = L.p;
@@ -424,7 +424,7 @@ __device__ __forceinline__ int qubit_of(int a, int rb) { return a < 5 ? rb + a :
 template <int MODE>
 __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_kernel(const __grid_constant__ BigLaunch L) {
     const int lane = threadIdx.x & 31;
-    const int64_t gw = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp_index();
     const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
     const int nin = L.n_in, b = L.b, RB = L.rb;
     const int r0 = L.w0 - b, r1 = L.w1 - b;  // register bits of the outer qubits to mix

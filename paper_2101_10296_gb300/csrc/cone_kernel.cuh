@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kRegBlock, GRAD ? (R <= 4 ? kGradMinBlocks : k
     constexpr int G_C = PC > 0 ? reg_group(PC, GRAD) : 0;
     const int NOUT = PC > 0 ? NOUT_C : reg_outputs(p, GRAD);
     const int G = PC > 0 ? G_C : reg_group(p, GRAD);
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_index();
     float2 *my_tab = s_tab + warp * (L.jpt * row);
     float2 *my_mix = s_tab + (kRegBlock / 32) * (L.jpt * row) + warp * (L.jpt * p);
     float *my_kp = reinterpret_cast<float *>(s_tab + (kRegBlock / 32) * (L.jpt * (row + p))) +
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kRegBlock, GRAD ? (R <= 4 ? kGradMinBlocks : k
     float *red = red_all + warp * (NOUT * G * 32);
     uint32_t *my_cone =
         reinterpret_cast<uint32_t *>(red_all + (kRegBlock / 32) * (NOUT * G * 32)) + warp * (reg_lane_words(p) * 32);
-    const int64_t gw = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int64_t gw = int64_t(blockIdx.x) * (kRegBlock / 32) + warp;
     const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
     const int64_t nblk = (L.n_points + L.jpt - 1) / L.jpt;
     const int64_t ntask = W.warps * nblk;

