@@ -507,6 +507,7 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
     pa.grad = grad;
     pa.terms = terms;
     pa.n_reps = d->n_cones;
+    pa.n_kpow = d->n_kpow;
     e = launch_prep(pa, s);
     qaoa_device_plan *dm = const_cast<qaoa_device_plan *>(d);
     dm->all_launches += 1;
@@ -729,6 +730,7 @@ extern "C" int qaoa_plan_upload(qaoa_plan *plan) {
     cudaGetDevice(&d->device);
     d->n_cones = int64_t(hc.size());
     d->cmax1 = cmax + 1;
+    for (const Cone &c : plan->cones) d->n_kpow = std::max(d->n_kpow, c.n_in + 1);
     d->n_big = n_big;
     plan->dev = d;
     cudaError_t e;

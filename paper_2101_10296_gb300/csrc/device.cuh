@@ -139,6 +139,7 @@ struct PrepArgs {
     double *grad;             // may be null
     double *terms;            // may be null
     int64_t n_reps;
+    int32_t n_kpow;           // kappa powers filled per row: what the plan's mixers read (<= kKpow)
 };
 
 // launchers (kernels.cu)

@@ -48,6 +48,7 @@ struct qaoa_device_plan {
     uint64_t *shell = nullptr;  // shell table (see DevCone)
     int32_t *status = nullptr;
     int32_t cmax1 = 1;
+    int32_t n_kpow = 3;  // kappa powers the kernels read: exponents up to the largest mixed set
     int64_t n_big = 0;
     int32_t points_per_task = 0;  // 0: default (see qaoa_tuning_t)
     int32_t blocks_per_sm = 0;

@@ -31,6 +31,7 @@
 // once; lane partial sums are reduced across the warp in FP32 and
 // accumulated across warps, cones and orbits in FP64 (atomicAdd).
 #include <algorithm>
+#include <cstdint>
 #include <map>
 #include <set>
 #include <mutex>
@@ -41,47 +42,72 @@
 namespace qaoa {
 namespace {
 
-__global__ void prep_kernel(const PrepArgs a) {
-    const int64_t tid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+// Per-call tables and output initialisation.  Bound: the FP64 pipe (two lanes
+// per clock and SM), and for small calls its latency, so the work is spread
+// over the SMs in blocks of one or two warps and a table row is cut into
+// `parts` segments while the rows alone would leave SMs idle.  The first
+// row_blocks blocks fill phase-table rows, the next mix_blocks the mixer
+// tables, the rest initialise the outputs.
+// Measured: the whole call of an 8x8 torus at p = 2, 128 points, energy 35 -> 17
+// us (256 rows of 24 entries had sat on one SM, 33 kappa powers each where 10
+// are read); the 48-graph mix at p = 1, 256 points 763 -> 749 us.
+constexpr int kPrepBlock = 64;
+
+__global__ void __launch_bounds__(kPrepBlock) prep_kernel(const PrepArgs a, int parts, int row_blocks, int mix_blocks) {
     const int64_t GP = int64_t(a.G) * a.P;
     const int p2 = 2 * a.p;
-    // one row per (graph, point, layer): exp(-i gamma c) for c = 0 .. cmax1-1 by the
-    // recurrence z_(c+1) = z_c exp(-i gamma) in FP64 (one sincos per row; after at most
-    // 64 steps its rounding error, ~1e-14, is far below the FP32 table's own)
-    for (int64_t r = tid; r < GP * a.p; r += stride) {
-        const int64_t l = r % a.p;
+    if (int(blockIdx.x) < row_blocks) {
+        // exp(-i gamma c) of one (graph, point, layer), c in the thread's segment: the segment's first
+        // entry directly, then the recurrence z_(c+1) = z_c exp(-i gamma) in FP64 (after at most 64
+        // steps its rounding error, ~1e-14, is far below the FP32 table's own)
+        const int64_t t = int64_t(blockIdx.x) * kPrepBlock + threadIdx.x;
+        const int64_t r = t / parts;
+        if (r >= GP * a.p) return;
+        const int part = int(t - r * parts);
         const int64_t gj = r / a.p;
+        const double gamma = a.params[gj * p2 + (r - gj * a.p)];
         double sn, cs;
-        sincos(a.params[gj * p2 + l], &sn, &cs);
+        sincos(gamma, &sn, &cs);
+        const int len = (a.cmax1 + parts - 1) / parts;
+        const int c0 = part * len, c1 = min(c0 + len, a.cmax1);
         float2 *row = a.lut + r * a.cmax1;
         double zr = 1.0, zi = 0.0;
-        for (int c = 0; c < a.cmax1; ++c) {
+        if (c0 > 0) {
+            sincos(gamma * double(c0), &zi, &zr);
+            zi = -zi;
+        }
+        for (int c = c0; c < c1; ++c) {
             row[c] = make_float2(float(zr), float(zi));
             const double nr = fma(zr, cs, zi * sn);  // (zr + i zi)(cos gamma - i sin gamma)
             zi = fma(zi, cs, -(zr * sn));
             zr = nr;
         }
+        return;
     }
-    for (int64_t i = tid; i < GP * a.p; i += stride) {
-        const int64_t gj = i / a.p, l = i % a.p;
+    const int64_t u = int64_t(int(blockIdx.x) - row_blocks) * kPrepBlock + threadIdx.x;
+    if (int(blockIdx.x) < row_blocks + mix_blocks) {
+        if (u >= GP * a.p) return;
+        const int64_t gj = u / a.p, l = u - gj * a.p;
         double sn, cs;
         sincos(a.params[gj * p2 + a.p + l], &sn, &cs);
         const bool flip = fabs(sn) > fabs(cs);
         const double tau = flip ? -cs / sn : sn / cs;
         const double k2 = flip ? sn * sn : cs * cs;
-        a.mix[i] = make_float2(float(tau), flip ? 1.f : 0.f);
+        a.mix[u] = make_float2(float(tau), flip ? 1.f : 0.f);
         double pw = 1.0;
-        for (int k = 0; k < kKpow; ++k) {
-            a.kpow[i * kKpow + k] = float(pw);
+        for (int k = 0; k < a.n_kpow; ++k) {
+            a.kpow[u * kKpow + k] = float(pw);
             pw *= k2;
         }
+        return;
     }
-    for (int64_t i = tid; i < GP; i += stride) a.energy[i] = a.half_edges[i / a.P];
+    const int64_t first = u - int64_t(mix_blocks) * kPrepBlock;
+    const int64_t stride = int64_t(int(gridDim.x) - row_blocks - mix_blocks) * kPrepBlock;
+    for (int64_t i = first; i < GP; i += stride) a.energy[i] = a.half_edges[i / a.P];
     if (a.grad)
-        for (int64_t i = tid; i < GP * p2; i += stride) a.grad[i] = 0.0;
+        for (int64_t i = first; i < GP * p2; i += stride) a.grad[i] = 0.0;
     if (a.terms)
-        for (int64_t i = tid; i < a.n_reps * a.P; i += stride) a.terms[i] = 0.0;
+        for (int64_t i = first; i < a.n_reps * a.P; i += stride) a.terms[i] = 0.0;
 }
 
 // C(z) for every z of one cone, through the same cut-word routine.
@@ -166,13 +192,18 @@ int smem_per_block(int blocks) {
 }
 
 cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s) {
-    // threads for the widest loop: table rows, gradient zeroing or term zeroing
-    int64_t work = int64_t(a.G) * a.P * 2 * a.p;
-    if (a.terms) work = std::max<int64_t>(work, a.n_reps * a.P);
-    int64_t blocks = (work + 255) / 256;
-    if (blocks < 1) blocks = 1;
-    if (blocks > 4096) blocks = 4096;
-    prep_kernel<<<int(blocks), 256, 0, s>>>(a);
+    const int64_t rows = int64_t(a.G) * a.P * a.p;
+    // segments per table row while rows x segments fit one block per SM
+    int parts = 1;
+    while (parts < 8 && rows * parts * 2 <= int64_t(sm_count()) * kPrepBlock) parts *= 2;
+    auto blocks = [](int64_t threads) { return (threads + kPrepBlock - 1) / kPrepBlock; };
+    const int64_t row_blocks = blocks(rows * parts), mix_blocks = blocks(rows);
+    int64_t out = int64_t(a.G) * a.P * (a.grad ? 2 * a.p : 1);
+    if (a.terms) out = std::max<int64_t>(out, a.n_reps * a.P);
+    const int64_t out_blocks = std::min<int64_t>(blocks(out), int64_t(sm_count()) * 8);
+    if (row_blocks + mix_blocks + out_blocks > INT32_MAX) return cudaErrorInvalidValue;
+    prep_kernel<<<int(row_blocks + mix_blocks + out_blocks), kPrepBlock, 0, s>>>(a, parts, int(row_blocks),
+                                                                                  int(mix_blocks));
     return cudaGetLastError();
 }
 

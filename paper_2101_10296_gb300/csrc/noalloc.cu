@@ -134,6 +134,7 @@ extern "C" int qaoa_energy_noalloc(const qaoa_plan *plan, int64_t n_points, cons
     pa.grad = nullptr;
     pa.terms = terms_dev;
     pa.n_reps = d->n_cones;
+    pa.n_kpow = d->n_kpow;
     e = launch_prep(pa, s);
     // register-resident cones: the depth-1 kernel where the plan has its list
     // (p = 1, no per-cone terms asked for), else the general register kernel
