@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -25,6 +26,62 @@ int cuda_fail(cudaError_t e, const char *what) {
     set_error(std::string(what) + ": " + cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? QAOA_E_OOM : QAOA_E_CUDA;
 }
+
+// Stream-ordered scratch of the calls comes from a memory pool of the library's
+// own, one per device.  A pool with release threshold 0 (the device's default
+// pool) gives all its memory back at every synchronisation, and mapping it again
+// cost the next call 0.2 ms (2.5 ms with large-state scratch); this one keeps up
+// to kPoolKeep bytes while the device holds an uploaded plan and gives them back
+// with the last.
+constexpr uint64_t kPoolKeep = uint64_t(2) << 30;
+constexpr int kPoolDevices = 64;
+struct DevicePool {
+    cudaMemPool_t pool = nullptr;
+    int64_t plans = 0;
+};
+std::mutex g_pool_mu;
+DevicePool g_pools[kPoolDevices];
+
+void pool_keep(cudaMemPool_t pool, uint64_t bytes) {
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &bytes);
+}
+
+// The device's pool for one more uploaded plan; null (the default pool serves) if
+// it cannot be made.
+cudaMemPool_t pool_retain(int dev) {
+    if (dev < 0 || dev >= kPoolDevices) return nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    DevicePool &d = g_pools[dev];
+    if (!d.pool) {
+        cudaMemPoolProps props;
+        std::memset(&props, 0, sizeof props);
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess) {
+            cudaGetLastError();
+            d.pool = nullptr;
+            return nullptr;
+        }
+    }
+    if (d.plans++ == 0) pool_keep(d.pool, kPoolKeep);
+    return d.pool;
+}
+
+void pool_release(int dev) {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    DevicePool &d = g_pools[dev];
+    if (--d.plans == 0) {
+        pool_keep(d.pool, 0);  // what is still in flight goes at the next synchronisation
+        cudaMemPoolTrimTo(d.pool, 0);
+    }
+}
+
+cudaError_t scratch_alloc(const qaoa_device_plan *d, void **ptr, size_t bytes, cudaStream_t s) {
+    return d->pool ? cudaMallocFromPoolAsync(ptr, bytes, d->pool, s) : cudaMallocAsync(ptr, bytes, s);
+}
+
+size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 void free_work(DevWork &w) {
     cudaFree(w.slot_cone);
@@ -393,18 +450,10 @@ namespace {
 // each wave streamed through the shape's pass list.
 cudaError_t run_big(const qaoa_device_plan *d, const qaoa_plan *plan, int64_t P, const double *params,
                     const float2 *lut, const float2 *mix, const float *kpow, double *energy, double *grad,
-                    double *terms, bool norm, cudaStream_t s) {
+                    double *terms, bool norm, float4 *cs, float2 *fa, cudaStream_t s) {
     qaoa_device_plan *dm = const_cast<qaoa_device_plan *>(d);
     const int p = plan->p;
-    float4 *cs = nullptr;
-    float2 *fa = nullptr;  // the adjoint's first-layer coefficient in hi + lo
-    cudaError_t e = cudaMallocAsync(&cs, size_t(plan->n_graphs) * P * p * sizeof(float4), s);
-    if (e != cudaSuccess) return e;
-    if (grad && (e = cudaMallocAsync(&fa, size_t(plan->n_graphs) * P * sizeof(float2), s)) != cudaSuccess) {
-        cudaFreeAsync(cs, s);
-        return e;
-    }
-    e = launch_big_prep(params, int64_t(plan->n_graphs) * P, p, cs, fa, s);
+    cudaError_t e = launch_big_prep(params, int64_t(plan->n_graphs) * P, p, cs, fa, s);
     dm->all_launches += 1;
     const bool g = grad != nullptr;
     const int grid = big_grid(g);
@@ -416,7 +465,7 @@ cudaError_t run_big(const qaoa_device_plan *d, const qaoa_plan *plan, int64_t P,
         const int64_t items = bs.ystart.back() * P;
         const int64_t wave = std::max<int64_t>(1, std::min<int64_t>(items, int64_t(d->big_budget) / block_bytes));
         float2 *scratch = nullptr;
-        e = cudaMallocAsync(&scratch, size_t(wave) * block_bytes, s);
+        e = scratch_alloc(d, reinterpret_cast<void **>(&scratch), size_t(wave) * block_bytes, s);
         if (e != cudaSuccess) break;
         BigLaunch B{};
         B.cones = d->cones;
@@ -457,8 +506,6 @@ cudaError_t run_big(const qaoa_device_plan *d, const qaoa_plan *plan, int64_t P,
         }
         cudaFreeAsync(scratch, s);
     }
-    cudaFreeAsync(cs, s);
-    if (fa) cudaFreeAsync(fa, s);
     return e;
 }
 
@@ -474,25 +521,24 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
     if (rc != QAOA_OK) return rc;
     const qaoa_device_plan *d = plan->dev;
     const int32_t G = plan->n_graphs, p = plan->p;
-    float2 *lut = nullptr, *mix = nullptr;
-    float *kpow = nullptr;
     if (take_fault(QAOA_FAULT_DEVICE_ALLOC)) {
         set_error("cudaMallocAsync: out of memory (injected by qaoa_inject_fault)");
         return QAOA_E_OOM;
     }
-    const size_t nlut = size_t(G) * n_points * p * d->cmax1;
-    const size_t nmix = size_t(G) * n_points * p;
-    cudaError_t e;
-    if ((e = cudaMallocAsync(&lut, nlut * sizeof(float2), s)) != cudaSuccess) return cuda_fail(e, "cudaMallocAsync");
-    if ((e = cudaMallocAsync(&mix, nmix * sizeof(float2), s)) != cudaSuccess) {
-        cudaFreeAsync(lut, s);
-        return cuda_fail(e, "cudaMallocAsync");
-    }
-    if ((e = cudaMallocAsync(&kpow, nmix * kKpow * sizeof(float), s)) != cudaSuccess) {
-        cudaFreeAsync(mix, s);
-        cudaFreeAsync(lut, s);
-        return cuda_fail(e, "cudaMallocAsync");
-    }
+    // one block: phase tables, mixer tables and, for large-state cones, their
+    // rotations and the adjoint's first-layer coefficient in hi + lo
+    const size_t rows = size_t(G) * size_t(n_points) * size_t(p);
+    const size_t lut_b = align256(rows * d->cmax1 * sizeof(float2)), mix_b = align256(rows * sizeof(float2));
+    const size_t kpow_b = align256(rows * kKpow * sizeof(float));
+    const size_t cs_b = d->big.empty() ? 0 : align256(rows * sizeof(float4));
+    const size_t fa_b = d->big.empty() || !grad ? 0 : size_t(G) * size_t(n_points) * sizeof(float2);
+    unsigned char *block = nullptr;
+    cudaError_t e = scratch_alloc(d, reinterpret_cast<void **>(&block), lut_b + mix_b + kpow_b + cs_b + fa_b, s);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync");
+    float2 *lut = reinterpret_cast<float2 *>(block), *mix = reinterpret_cast<float2 *>(block + lut_b);
+    float *kpow = reinterpret_cast<float *>(block + lut_b + mix_b);
+    float4 *cs = cs_b ? reinterpret_cast<float4 *>(block + lut_b + mix_b + kpow_b) : nullptr;
+    float2 *fa = fa_b ? reinterpret_cast<float2 *>(block + lut_b + mix_b + kpow_b + cs_b) : nullptr;
     PrepArgs pa;
     pa.params = params;
     pa.G = G;
@@ -557,7 +603,7 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
         int64_t grid = std::min<int64_t>(tuned_grid(d, reg_p1_grid(grad != nullptr, smem)), (tasks + 3) / 4);
         e = launch_reg_p1(L, grad != nullptr, int(std::max<int64_t>(grid, 1)), s);
         dm->all_launches += 1;
-        if (e == cudaSuccess && !d->big.empty()) e = run_big(d, plan, n_points, params, lut, mix, kpow, energy, grad, terms, norm, s);
+        if (e == cudaSuccess && !d->big.empty()) e = run_big(d, plan, n_points, params, lut, mix, kpow, energy, grad, terms, norm, cs, fa, s);
     } else if (e == cudaSuccess) {
         RegLaunch L;
         L.n_points = n_points;
@@ -576,15 +622,13 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
         L.work = as_reg(d, d->reg[rg - 4]);
         if (L.work.warps > 0) e = launch_reg(d, L, g, rg, d->points_per_task, s);
         if (L.work.warps > 0) dm->all_launches += 1;
-        if (e == cudaSuccess && !d->big.empty()) e = run_big(d, plan, n_points, params, lut, mix, kpow, energy, grad, terms, norm, s);
+        if (e == cudaSuccess && !d->big.empty()) e = run_big(d, plan, n_points, params, lut, mix, kpow, energy, grad, terms, norm, cs, fa, s);
     }
     if (ev0) {
         cudaEventRecord(ev1, s);
         dm->events.emplace_back(ev0, ev1);
     }
-    cudaFreeAsync(kpow, s);
-    cudaFreeAsync(mix, s);
-    cudaFreeAsync(lut, s);
+    cudaFreeAsync(block, s);
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     return QAOA_OK;
 }
@@ -613,6 +657,7 @@ extern "C" void qaoa_device_release(qaoa_plan *plan) {
         cudaEventDestroy(pr.second);
     }
     if (cur >= 0) cudaSetDevice(cur);
+    if (d->pool) pool_release(d->device);
     delete d;
     plan->dev = nullptr;
 }
@@ -728,6 +773,7 @@ extern "C" int qaoa_plan_upload(qaoa_plan *plan) {
         shape->ystart.push_back(shape->ystart.back() + c.n_blocks);
     }
     cudaGetDevice(&d->device);
+    d->pool = pool_retain(d->device);
     d->n_cones = int64_t(hc.size());
     d->cmax1 = cmax + 1;
     for (const Cone &c : plan->cones) d->n_kpow = std::max(d->n_kpow, c.n_in + 1);
@@ -848,8 +894,10 @@ extern "C" int qaoa_norms(const qaoa_plan *plan, int64_t n_points, const double 
         return QAOA_E_INVALID;
     }
     const cudaStream_t s = (cudaStream_t)stream;
+    int up = ensure_uploaded(plan);
+    if (up != QAOA_OK) return up;
     double *scratch = nullptr;  // the energy output of the identity observable, unused
-    cudaError_t e = cudaMallocAsync(&scratch, size_t(plan->n_graphs) * size_t(n_points) * sizeof(double), s);
+    cudaError_t e = scratch_alloc(plan->dev, reinterpret_cast<void **>(&scratch), size_t(plan->n_graphs) * size_t(n_points) * sizeof(double), s);
     if (e != cudaSuccess) {
         set_error(std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
         return e == cudaErrorMemoryAllocation ? QAOA_E_OOM : QAOA_E_CUDA;

@@ -34,6 +34,7 @@ struct BigShape {
 
 struct qaoa_device_plan {
     int device = -1;
+    cudaMemPool_t pool = nullptr;  // the device's scratch pool (capi.cu), or null: the default pool
     qaoa::DevCone *cones = nullptr;
     int64_t n_cones = 0;
     // Work lists with 4 and 5 register qubits per thread: the energy takes 5, the

@@ -145,10 +145,20 @@ def inject_fault(kind, count=1):
     _check(lib().qaoa_inject_fault(kind, count))
 
 
+_torch = None
+
+
+def _t():
+    """torch, imported on the first call that needs it (planning does not)."""
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch
+
+
 def _stream_handle(stream=None):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    return stream.cuda_stream if stream is not None else _t().cuda.current_stream().cuda_stream
 
 
 class Plan:
@@ -192,6 +202,7 @@ class Plan:
         self.p = p
         self.n_graphs = len(graphs)
         self.n_edges = [int(r.shape[0]) for r in rows]
+        self._n_reps = None  # filled on first use: a plan's representatives never change
 
     def close(self):
         if getattr(self, "_h", None) and self._h.value:
@@ -208,6 +219,11 @@ class Plan:
         i = PlanInfo()
         _check(lib().qaoa_plan_info(self._h, C.byref(i)))
         return {k: getattr(i, k) for k, _ in PlanInfo._fields_}
+
+    def _reps_count(self):
+        if self._n_reps is None:
+            self._n_reps = self.info()["n_reps"]
+        return self._n_reps
 
     def orbits(self, graph=0):
         oid = np.zeros(self.n_edges[graph], dtype=np.int32)
@@ -296,7 +312,7 @@ class Plan:
         return out
 
     def _params(self, params):
-        import torch
+        torch = _t()
         if not (isinstance(params, torch.Tensor) and params.is_cuda and params.dtype == torch.float64):
             raise TypeError("params must be a CUDA float64 tensor")
         # device pointers must be on the current device (the library checks that the
@@ -312,24 +328,23 @@ class Plan:
 
     def energy(self, params, terms=False, stream=None):
         """E[g, j] for params [G, P, 2p] (CUDA float64); optionally <ZZ> per rep."""
-        import torch
+        torch = _t()
         params = self._params(params)
-        G, P = params.shape[0], params.shape[1]
+        G, P, _ = params.shape
         e = torch.empty(G, P, dtype=torch.float64, device=params.device)
-        t = torch.empty(self.info()["n_reps"], P, dtype=torch.float64, device=params.device) if terms else None
-        _check(lib().qaoa_energy(self._h, P, C.c_void_p(params.data_ptr()), C.c_void_p(e.data_ptr()),
-                                 C.c_void_p(t.data_ptr()) if terms else None, _stream_handle(stream)))
+        t = torch.empty(self._reps_count(), P, dtype=torch.float64, device=params.device) if terms else None
+        _check(lib().qaoa_energy(self._h, P, params.data_ptr(), e.data_ptr(), t.data_ptr() if terms else None,
+                                 _stream_handle(stream)))
         return (e, t) if terms else e
 
     def norms(self, params, stream=None):
         """sum_z |psi_z|^2 of every representative's cone state at every point,
         [n_reps, P] (1 up to the FP32 state's rounding; a diagnostic)."""
-        import torch
+        torch = _t()
         params = self._params(params)
         P = params.shape[1]
-        out = torch.empty(self.info()["n_reps"], P, dtype=torch.float64, device=params.device)
-        _check(lib().qaoa_norms(self._h, P, C.c_void_p(params.data_ptr()), C.c_void_p(out.data_ptr()),
-                                _stream_handle(stream)))
+        out = torch.empty(self._reps_count(), P, dtype=torch.float64, device=params.device)
+        _check(lib().qaoa_norms(self._h, P, params.data_ptr(), out.data_ptr(), _stream_handle(stream)))
         return out
 
     def energy_noalloc(self, params, out=None, terms=None, stream=None):
@@ -339,9 +354,9 @@ class Plan:
         are allocated here by torch only when not given.  The plan must have
         been uploaded (``upload()``).
         """
-        import torch
+        torch = _t()
         params = self._params(params)
-        G, P = params.shape[0], params.shape[1]
+        G, P, _ = params.shape
         if out is None:
             out = torch.empty(G, P, dtype=torch.float64, device=params.device)
 
@@ -357,23 +372,21 @@ class Plan:
 
         _need(out, (G, P), "out")
         if terms is not None:
-            _need(terms, (self.info()["n_reps"], P), "terms")
-        _check(lib().qaoa_energy_noalloc(self._h, P, C.c_void_p(params.data_ptr()), C.c_void_p(out.data_ptr()),
-                                         C.c_void_p(terms.data_ptr()) if terms is not None else None,
-                                         _stream_handle(stream)))
+            _need(terms, (self._reps_count(), P), "terms")
+        _check(lib().qaoa_energy_noalloc(self._h, P, params.data_ptr(), out.data_ptr(),
+                                         terms.data_ptr() if terms is not None else None, _stream_handle(stream)))
         return out
 
     def energy_grad(self, params, terms=False, stream=None):
         """(E[g, j], dE/dtheta[g, j, 2p]) by the adjoint kernels."""
-        import torch
+        torch = _t()
         params = self._params(params)
-        G, P = params.shape[0], params.shape[1]
+        G, P, p2 = params.shape
         e = torch.empty(G, P, dtype=torch.float64, device=params.device)
-        g = torch.empty(G, P, 2 * self.p, dtype=torch.float64, device=params.device)
-        t = torch.empty(self.info()["n_reps"], P, dtype=torch.float64, device=params.device) if terms else None
-        _check(lib().qaoa_energy_grad(self._h, P, C.c_void_p(params.data_ptr()), C.c_void_p(e.data_ptr()),
-                                      C.c_void_p(g.data_ptr()), C.c_void_p(t.data_ptr()) if terms else None,
-                                      _stream_handle(stream)))
+        g = torch.empty(G, P, p2, dtype=torch.float64, device=params.device)
+        t = torch.empty(self._reps_count(), P, dtype=torch.float64, device=params.device) if terms else None
+        _check(lib().qaoa_energy_grad(self._h, P, params.data_ptr(), e.data_ptr(), g.data_ptr(),
+                                      t.data_ptr() if terms else None, _stream_handle(stream)))
         return (e, g, t) if terms else (e, g)
 
     def set_tuning(self, points_per_task=0, blocks_per_sm=0, big_scratch_bytes=0, reg_bits_grad=0, chunk_window=0):
