@@ -288,13 +288,14 @@ int build_depth2_work(const std::vector<DevCone> &hc, const std::vector<int32_t>
 
 // The depth-1 kernel's list (every cone with inner part {u, v}, mixed by the
 // only layer): per graph, the shell blocks of its cones back to back, each
-// as (c_0 | c_1 << 8 | c_2 << 16 | c_3 << 24, W) with c_a the cut value of
+// as (count bytes, W), with byte a the cut value (scaled, see RegWork) of
 // amplitude a = z_u + 2 z_v of the block (up to the relabelling below) and
 // W = +-multiplicity x orbit size x 2^-n rounded once to float; slot s of a
 // graph takes its blocks 16 s .. 16 s + 15, and every graph starts on a
 // fresh warp (padding: zero weight).
 int build_p1_work(const std::vector<DevCone> &hc, const std::vector<uint64_t> &shell_tab,
-                  const std::vector<int32_t> &idx, DevWork &w) {
+                  const std::vector<int32_t> &idx, int cmax1, DevWork &w) {
+    const int unit = p1_row_bytes(cmax1) == kP1RowLarge ? 1 : 4;  // of the count bytes
     std::vector<int32_t> order(idx);
     std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return hc[a].graph < hc[b].graph; });
     std::vector<uint2> blocks;  // flat, graph by graph, each graph padded to 32 slots
@@ -326,7 +327,7 @@ int build_p1_work(const std::vector<DevCone> &hc, const std::vector<uint64_t> &s
                     }
                 }
                 uint32_t cnt = 0;
-                for (int a = 0; a < 4; ++a) cnt |= uint32_t(c[a ^ f]) << (8 * a);
+                for (int a = 0; a < 4; ++a) cnt |= uint32_t(c[a ^ f] * unit) << (8 * a);
                 const float wf = float(double(mult) * scale) * ((f == 1 || f == 2) ? -1.f : 1.f);
                 uint32_t bits;
                 std::memcpy(&bits, &wf, sizeof bits);
@@ -343,16 +344,19 @@ int build_p1_work(const std::vector<DevCone> &hc, const std::vector<uint64_t> &s
     w.warps = slots / 32;
     w.n = int32_t(order.size());
     if (slots == 0) return QAOA_OK;
-    // records [k][slot]: block k of slot s is flat block 16 s + k
-    std::vector<uint2> rec(blocks.size());
+    // records [q][slot]: blocks 2q and 2q + 1 of slot s are flat blocks 16 s + 2q and the next
+    std::vector<uint4> rec(blocks.size() / 2);
     for (int64_t sl = 0; sl < slots; ++sl)
-        for (int k = 0; k < kP1Blocks; ++k)
-            rec[size_t(k) * size_t(slots) + size_t(sl)] = blocks[size_t(sl) * kP1Blocks + size_t(k)];
+        for (int q = 0; q < kP1Blocks / 2; ++q) {
+            const uint2 &a = blocks[size_t(sl) * kP1Blocks + size_t(2 * q)];
+            const uint2 &b = blocks[size_t(sl) * kP1Blocks + size_t(2 * q + 1)];
+            rec[size_t(q) * size_t(slots) + size_t(sl)] = make_uint4(a.x, b.x, a.y, b.y);
+        }
     cudaError_t e;
     if ((e = cudaMalloc(&w.warp_graph, wgraph.size() * sizeof(int32_t))) != cudaSuccess ||
-        (e = cudaMalloc(&w.rec_cw, rec.size() * sizeof(uint2))) != cudaSuccess)
+        (e = cudaMalloc(&w.rec_cw, rec.size() * sizeof(uint4))) != cudaSuccess)
         return cuda_fail(e, "cudaMalloc");
-    e = cudaMemcpy(w.rec_cw, rec.data(), rec.size() * sizeof(uint2), cudaMemcpyHostToDevice);
+    e = cudaMemcpy(w.rec_cw, rec.data(), rec.size() * sizeof(uint4), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(w.warp_graph, wgraph.data(), wgraph.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy");
@@ -578,29 +582,30 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
         L.terms = nullptr;
         L.status = d->status;
         L.work = as_reg(d, d->reg_p1);
-        // points per warp task: as many phase tables as leave room for the
-        // resident blocks the kernel is sized for (a tuned value is held to
-        // the kernel's shared-memory limit), halved while the tasks would not
-        // give every SM 16 warps
+        // points per warp task: as many phase tables as leave room for
+        // kP1PointBlocks resident blocks (a tuned value is held to the kernel's
+        // shared-memory limit), halved while the tasks would not give every SM
+        // 16 warps, and evened out over the tasks
         {
             const bool g = grad != nullptr;
-            const int64_t row = int64_t(d->cmax1 + 1) * int64_t(sizeof(float2));
+            const int64_t row = int64_t(p1_row_bytes(d->cmax1)) + int64_t(sizeof(float2));
             const int64_t fixed = int64_t(reg_p1_smem_bytes(0, d->cmax1, g)) / (kRegBlock / 32);
-            const int blocks = g ? kP1GradMinBlocks : kP1EnergyMinBlocks;
-            const int64_t fit = (int64_t(smem_per_block(blocks)) / (kRegBlock / 32) - fixed) / row;
+            const int64_t fit = (int64_t(smem_per_block(kP1PointBlocks)) / (kRegBlock / 32) - fixed) / row;
             const int64_t cap = (int64_t(kRegMaxSmem) / (kRegBlock / 32) - fixed) / row;
             int64_t jpt = d->points_per_task;
             if (jpt <= 0) {
                 jpt = std::min<int64_t>(32, std::max<int64_t>(1, fit));
                 while (jpt > 1 && L.work.warps * ((n_points + jpt - 1) / jpt) < int64_t(sm_count()) * 16)
                     jpt = (jpt + 1) / 2;
+                const int64_t nblk = (n_points + jpt - 1) / jpt;
+                jpt = (n_points + nblk - 1) / nblk;
             }
             jpt = std::max<int64_t>(1, std::min<int64_t>(jpt, cap));
             L.jpt = int32_t(std::min<int64_t>(jpt, n_points));
         }
         const size_t smem = reg_p1_smem_bytes(L.jpt, d->cmax1, grad != nullptr);
         const int64_t tasks = L.work.warps * ((n_points + L.jpt - 1) / L.jpt);
-        int64_t grid = std::min<int64_t>(tuned_grid(d, reg_p1_grid(grad != nullptr, smem)), (tasks + 3) / 4);
+        int64_t grid = std::min<int64_t>(tuned_grid(d, reg_p1_grid(grad != nullptr, d->cmax1, smem)), (tasks + 3) / 4);
         e = launch_reg_p1(L, grad != nullptr, int(std::max<int64_t>(grid, 1)), s);
         dm->all_launches += 1;
         if (e == cudaSuccess && !d->big.empty()) e = run_big(d, plan, n_points, params, lut, mix, kpow, energy, grad, terms, norm, cs, fa, s);
@@ -818,7 +823,7 @@ extern "C" int qaoa_plan_upload(qaoa_plan *plan) {
     // part): the depth-1 kernel's list
     bool p1 = plan->p == 1 && !reg_idx.empty();
     for (int32_t i : reg_idx) p1 = p1 && hc[size_t(i)].n_in == 2 && hc[size_t(i)].k[0] == 2;
-    if (rc == QAOA_OK && p1) rc = build_p1_work(hc, shell_tab, reg_idx, d->reg_p1);
+    if (rc == QAOA_OK && p1) rc = build_p1_work(hc, shell_tab, reg_idx, d->cmax1, d->reg_p1);
     if (rc == QAOA_OK) {
         std::vector<double> half(size_t(plan->n_graphs));
         for (int32_t g = 0; g < plan->n_graphs; ++g) half[g] = 0.5 * double(plan->weight_sum[g]);

@@ -98,7 +98,7 @@ struct RegWork {
     const void *rec_hi = nullptr;         // slot records (above)
     const uint32_t *rec_cnt = nullptr;
     const float *rec_wk = nullptr;
-    const uint2 *rec_cw = nullptr;        // depth-1 work lists: per block the four cut values and the multiplicity
+    const uint4 *rec_cw = nullptr;        // depth-1 work lists: cut values and weights of two blocks
     int32_t n_cones = 0;
     int64_t slots = 0;                    // slots per point (with padding; a multiple of 32)
     int64_t warps = 0;                    // warps per point
@@ -207,26 +207,37 @@ constexpr int kRegKpow = 10;
 __host__ __device__ constexpr int reg_lane_words(int p) { return 3 + 2 * p; }
 // Depth-1 kernel (p1_kernel.cu): shell blocks per thread, and the resident
 // blocks per SM its register allocation is sized for.  Its work lists hold
-// per graph the shell blocks of all the graph's cones back to back, block k
-// of slot s as rec_cw[k * slots + s] = (c_0 | c_1 << 8 | c_2 << 16 | c_3 <<
-// 24, bits of W), c_a the cut value of amplitude a = z_u + 2 z_v and W the
-// block's multiplicity x orbit size x 2^-n; the amplitudes may be relabelled
-// by X_u, X_v or both (a -> a xor f), with W negated for a single flip, so
-// that c_0 is the middle one of the four; warp_graph as for the other lists.
+// per graph the shell blocks of all the graph's cones back to back, 16 to a
+// slot; rec_cw[q * slots + s] holds blocks 2q and 2q + 1 of slot s: their count
+// bytes (the cut value c_a of amplitude a = z_u + 2 z_v in byte a, scaled by 4
+// unless a cone has 64 cut bits), then their weights W = multiplicity x orbit
+// size x 2^-n; the amplitudes may be relabelled by X_u, X_v or both (a -> a xor
+// f), with W negated for a single flip, so that c_0 is the middle one of the
+// four; warp_graph as for the other lists.
 constexpr int kP1Blocks = 16;
-constexpr int kP1GradMinBlocks = 6;
-constexpr int kP1EnergyMinBlocks = 8;
-// Dynamic shared memory of a depth-1 block: per warp jpt phase tables, jpt
-// (tau, kappa^4) pairs, the records of its 32 slots and the reduction buffer.
+// Blocks per SM of the registers, and of the shared memory for the points of a
+// task.  Measured on the 48-graph mix at 256 points, adjoint: 4, 5, 6 and 8
+// blocks of registers 750, 736, 728 and 713 us, then 12 points per task (room
+// for six blocks) instead of 4: 691 us; energy 361, 350, 347 and 351 us.
+constexpr int kP1GradMinBlocks = 8;
+constexpr int kP1EnergyMinBlocks = 6;
+constexpr int kP1PointBlocks = 6;
 // Points per reduction group of the depth-1 kernel (see reg_flush): four for
 // the adjoint, whose three outputs would otherwise take 3 KB per warp
 __host__ __device__ constexpr int reg_p1_group(bool grad) { return grad ? 4 : 8; }
+// Bytes of a point's phase-table row in shared memory (see p1_kernel.cu).
+constexpr int kP1RowSmall = 256, kP1RowMid = 512, kP1RowLarge = 544;
+__host__ __device__ constexpr int p1_row_bytes(int cmax1) {
+    return cmax1 <= 32 ? kP1RowSmall : cmax1 <= 64 ? kP1RowMid : kP1RowLarge;
+}
+// Dynamic shared memory of a depth-1 block: per warp jpt phase tables and (tau,
+// kappa^4) pairs, the records of its 32 slots and the reduction buffer.
 inline size_t reg_p1_smem_bytes(int jpt, int cmax1, bool grad) {
     return size_t(kRegBlock / 32) *
-           (size_t(jpt) * (cmax1 + 1) * sizeof(float2) + size_t(kP1Blocks) * 32 * sizeof(uint2) +
+           (size_t(jpt) * (p1_row_bytes(cmax1) + sizeof(float2)) + size_t(kP1Blocks / 2) * 32 * sizeof(uint4) +
             size_t(reg_outputs(1, grad)) * reg_p1_group(grad) * 32 * sizeof(float));
 }
-int reg_p1_grid(bool grad, size_t smem);
+int reg_p1_grid(bool grad, int cmax1, size_t smem);
 cudaError_t reg_p1_prepare();
 cudaError_t launch_reg_p1(const RegLaunch &a, bool grad, int grid, cudaStream_t s);
 

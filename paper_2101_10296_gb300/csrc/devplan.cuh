@@ -14,7 +14,7 @@ struct DevWork {
     void *rec_hi = nullptr;         // [S][slots] cut words (uint32 or uint64, see RegWork)
     uint32_t *rec_cnt = nullptr;    // depth-2 lists: [2][S][slots] cut values, one byte per amplitude
     float *rec_wk = nullptr;        // [S][slots] block multiplicities
-    uint2 *rec_cw = nullptr;        // depth-1 lists: [kP1Blocks][slots] cut values and multiplicity
+    uint4 *rec_cw = nullptr;        // depth-1 lists: [kP1Blocks / 2][slots] cut values and weights of two blocks
     int64_t slots = 0, warps = 0;
     int32_t n = 0;
 };

@@ -143,7 +143,7 @@ extern "C" int qaoa_energy_noalloc(const qaoa_plan *plan, int64_t n_points, cons
         L.work = reg_work(d, d->reg_p1);
         L.n_points = n_points;
         L.p = 1;
-        const int64_t row = int64_t(d->cmax1 + 1) * int64_t(sizeof(float2));
+        const int64_t row = int64_t(p1_row_bytes(d->cmax1)) + int64_t(sizeof(float2));
         const int64_t fixed = int64_t(reg_p1_smem_bytes(0, d->cmax1, false)) / (kRegBlock / 32);
         const int64_t fit = (int64_t(kRegMaxSmem) / (kRegBlock / 32) - fixed) / row;
         L.jpt = int32_t(std::min<int64_t>(std::min<int64_t>(8, std::max<int64_t>(1, fit)), n_points));
@@ -157,7 +157,7 @@ extern "C" int qaoa_energy_noalloc(const qaoa_plan *plan, int64_t n_points, cons
         L.status = d->status;
         const size_t smem = reg_p1_smem_bytes(L.jpt, d->cmax1, false);
         const int64_t tasks = L.work.warps * ((n_points + L.jpt - 1) / L.jpt);
-        const int64_t grid = std::min<int64_t>(reg_p1_grid(false, smem), (tasks + 3) / 4);
+        const int64_t grid = std::min<int64_t>(reg_p1_grid(false, d->cmax1, smem), (tasks + 3) / 4);
         e = launch_reg_p1(L, false, int(std::max<int64_t>(grid, 1)), s);
     } else if (e == cudaSuccess && d->reg[kRegBitsEnergy - 4].warps > 0) {
         RegLaunch L;

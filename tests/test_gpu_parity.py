@@ -959,6 +959,38 @@ def test_adjoint_register_widths_match_oracle(q, graph, p, signs):
     assert plan.device_status() == 0
 
 
+@pytest.mark.parametrize("P", [1, 17])
+@pytest.mark.parametrize("leaves,weight", [(3, 10), (31, 1), (4, 8), (9, 7), (8, 8), (9, -7)],
+                         ids=["30-bits", "31-bits", "32-bits", "63-bits", "64-bits", "signed-63-bits"])
+def test_depth1_kernel_table_rows(q, leaves, weight, P):
+    """Depth-1 plans at the edges of the kernel's three table-row layouts (up to 31, up to 63 and 64
+    cut bits): energies and gradients against the FP64 oracle."""
+    n, edges = I.star(leaves)
+    w = np.full(len(edges), weight)
+    th = I.draw_params(1, P, 5)
+    plan = q.Plan((n, edges), 1, weights=[w])
+    assert plan.info()["depth1_kernel"] == 1
+    e, g = plan.energy_grad(_params(th))
+    e2 = plan.energy(_params(th))
+    scale = abs(weight) * len(edges)
+    for j in {0, P - 1}:
+        # every edge of a star is equivalent: the first edge's cone, a star of `leaves` leaves
+        if leaves < 20:
+            verts, _, ledges = O.lightcone(n, edges, edges[0], 1)
+            val, der = O.term_grad_adjoint(len(verts), ledges, th[j], 1, O.cone_weights(edges, w, verts, ledges))
+            eref, gref = scale * np.sign(weight) * val, scale * np.sign(weight) * der
+        else:
+            gam, bet = th[j]
+            h = 1e-6
+            f = lambda a, b: len(edges) * O.closed_form_p1_term(n, edges, edges[0], a, b)
+            eref = f(gam, bet)
+            gref = np.array([f(gam + h, bet) - f(gam - h, bet), f(gam, bet + h) - f(gam, bet - h)]) / (2 * h)
+        assert abs(e.cpu().numpy()[0, j] - eref) <= 1e-6 * scale
+        assert abs(e2.cpu().numpy()[0, j] - eref) <= 1e-6 * scale
+        _check_grad(g.cpu().numpy()[0, j], gref, energy=scale)
+    assert plan.device_status() == 0
+
+
 @pytest.mark.parametrize("P", [1, 33])
 @pytest.mark.parametrize("graph,weight", [
     ((2, np.array([[0, 1]])), 1), (I.path(5), 1), (I.star(5), 1), (I.complete(4), 1), (I.cycle(11), 3),
