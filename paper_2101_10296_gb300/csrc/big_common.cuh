@@ -19,11 +19,17 @@ __device__ __forceinline__ float2 unrot(float2 me, float2 o, float4 cs) {
                        fmaf(cs.x, me.y, fmaf(cs.y, o.x, fmaf(cs.z, me.y, cs.w * o.x))));
 }
 
+// Warp sum in FP32 (every lane gets it).
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    return v;
+}
+
 // Warp sum in FP32, then one FP64 atomic into base[idx] (energies and terms,
 // whose sums do not cancel).
 __device__ __forceinline__ void add_gp(float v, double *base, int64_t idx) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    v = warp_sum(v);
     if ((threadIdx.x & 31) == 0) atomicAdd(base + idx, double(v));
 }
 

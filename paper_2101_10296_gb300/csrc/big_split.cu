@@ -38,6 +38,7 @@
 
 #include "big.cuh"
 #include "big_common.cuh"
+#include "packed.cuh"
 
 namespace qaoa {
 namespace {
@@ -160,260 +161,389 @@ __device__ __forceinline__ void first_mix_lanes(float2 (&x)[NR], int nb, const F
     }
 }
 
-// exp(-i beta X) on register qubits [0, nbits) (nbits <= log2 NR).
-template <int NR>
-__device__ __forceinline__ void mix_regs(float2 (&x)[NR], int nbits, float4 cs) {
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return uint32_t(__cvta_generic_to_shared(p)); }
+
+// ---------------------------------------------------------------- core pass
+// The tile in packed FP32x2 pairs (packed.cuh): C2 number h holds registers h
+// and h + NR/2, every operation of the sweep is one instruction for both, and
+// the highest register qubit's partner is the other half.  Sums that run over
+// the registers in order (the observable, the derivative terms) take the lower
+// halves first, then the upper ones.
+
+// c me - i s o (rot) or c me + i s o (unrot), see big_common.cuh
+template <bool INV>
+__device__ __forceinline__ C2 rot2(const C2 &me, const C2 &o, float4 cs) {
+    const float s = INV ? -cs.y : cs.y, w = INV ? -cs.w : cs.w;
+    return C2{fma2(splat(cs.x), me.r, fma2(splat(s), o.i, fma2(splat(cs.z), me.r, mul2(splat(w), o.i)))),
+              fma2(splat(cs.x), me.i, fma2(splat(-s), o.r, fma2(splat(cs.z), me.i, mul2(splat(-w), o.r))))};
+}
+
+// fmix on two amplitudes
+template <bool B, bool INV, bool LO>
+__device__ __forceinline__ C2 fmix2(const C2 &me, const C2 &o, float a, float alo) {
+    const P2 oi = INV ? neg(o.i) : o.i, nor = INV ? o.r : neg(o.r);  // -i o, or i o
+    if (!B) {
+        const P2 ox = LO ? fma2(splat(alo), oi, me.r) : me.r, oy = LO ? fma2(splat(alo), nor, me.i) : me.i;
+        return C2{fma2(splat(a), oi, ox), fma2(splat(a), nor, oy)};
+    }
+    const P2 px = LO ? fma2(splat(alo), me.r, oi) : oi, py = LO ? fma2(splat(alo), me.i, nor) : nor;
+    return C2{fma2(splat(a), me.r, px), fma2(splat(a), me.i, py)};
+}
+
+// op(me, partner) on register qubit q of a tile
+template <int NP, class F>
+__device__ __forceinline__ void on_reg(C2 (&x)[NP], int q, F &&op) {
+    if ((1 << q) == NP) {
 #pragma unroll
-    for (int rb = 0; (1 << rb) < NR; ++rb) {
-        if (rb < nbits) {
+        for (int h = 0; h < NP; ++h) x[h] = op(x[h], swap(x[h]));
+    } else {
 #pragma unroll
-            for (int i = 0; i < NR; ++i) {
-                if (i & (1 << rb)) continue;
-                const int i2 = i | (1 << rb);
-                const float2 a = x[i], bb = x[i2];
-                x[i] = rot(a, bb, cs);
-                x[i2] = rot(bb, a, cs);
-            }
+        for (int h = 0; h < NP; ++h) {
+            if (h & (1 << q)) continue;
+            const int j = h | (1 << q);
+            const C2 u = x[h], v = x[j];
+            x[h] = op(u, v);
+            x[j] = op(v, u);
         }
     }
 }
 
-// exp(-i beta X) on lane bits [0, nb).
-template <int NR>
-__device__ __forceinline__ void mix_lanes(float2 (&x)[NR], int nb, float4 cs) {
-    for (int lb = 0; lb < nb; ++lb) {
-        const int m = 1 << lb;
+// op on register qubits [0, nr) and lane qubits [0, nl)
+template <int NP, class F>
+__device__ __forceinline__ void on_qubits(C2 (&x)[NP], int nr, int nl, F &&op) {
 #pragma unroll
-        for (int i = 0; i < NR; ++i) {
-            float2 o;
-            o.x = __shfl_xor_sync(kFull, x[i].x, m);
-            o.y = __shfl_xor_sync(kFull, x[i].y, m);
-            x[i] = rot(x[i], o, cs);
-        }
+    for (int q = 0; (1 << q) <= NP; ++q)
+        if (q < nr) on_reg<NP>(x, q, op);
+#pragma unroll 1
+    for (int lb = 0; lb < nl; ++lb) {
+#pragma unroll
+        for (int h = 0; h < NP; ++h) x[h] = op(x[h], shfl_xor(x[h], 1 << lb));
     }
 }
 
-// Adjoint step of a mixer on register qubits [0, nbits): adds
-// Im<r|X_q|x> for each (one qubit's terms at a time into the compensated
-// sum), then applies exp(+i beta X) to both states.
-template <int NR>
-__device__ __forceinline__ void unmix_regs_d(float2 (&x)[NR], float2 (&r)[NR], int nbits, float4 cs, Dfl &acc) {
-#pragma unroll
-    for (int rb = 0; (1 << rb) < NR; ++rb) {
-        if (rb < nbits) {
-            float d = 0.f;
-#pragma unroll
-            for (int i = 0; i < NR; ++i) {
-                if (i & (1 << rb)) continue;
-                const int i2 = i | (1 << rb);
-                const float2 a = x[i], bb = x[i2], ra = r[i], rbv = r[i2];
-                d += imconj(ra, bb) + imconj(rbv, a);
-                x[i] = unrot(a, bb, cs);
-                x[i2] = unrot(bb, a, cs);
-                r[i] = unrot(ra, rbv, cs);
-                r[i2] = unrot(rbv, ra, cs);
-            }
-            dfl_add(acc, d);
-        }
-    }
+template <int NP, bool INV, bool LO>
+__device__ __forceinline__ void first_mix2(C2 (&x)[NP], int nr, int nl, const FirstMix &f) {
+    if (__any_sync(kFull, f.b))  // the same in every lane: the vote tells the compiler
+        on_qubits<NP>(x, nr, nl, [&](const C2 &u, const C2 &v) { return fmix2<true, INV, LO>(u, v, f.a, f.alo); });
+    else
+        on_qubits<NP>(x, nr, nl, [&](const C2 &u, const C2 &v) { return fmix2<false, INV, LO>(u, v, f.a, f.alo); });
 }
 
-template <int NR>
-__device__ __forceinline__ void unmix_lanes_d(float2 (&x)[NR], float2 (&r)[NR], int nb, float4 cs, Dfl &acc) {
-    for (int lb = 0; lb < nb; ++lb) {
-        const int m = 1 << lb;
-        float d = 0.f;
+// Im<r|X_q|x> over register qubit q: the pairs' terms in register order.
+template <int NP>
+__device__ __forceinline__ float xterm_reg(const C2 (&x)[NP], const C2 (&r)[NP], int q) {
+    float d = 0.f;
+    if ((1 << q) == NP) {
 #pragma unroll
-        for (int i = 0; i < NR; ++i) {
-            float2 xo, ro;
-            xo.x = __shfl_xor_sync(kFull, x[i].x, m);
-            xo.y = __shfl_xor_sync(kFull, x[i].y, m);
-            ro.x = __shfl_xor_sync(kFull, r[i].x, m);
-            ro.y = __shfl_xor_sync(kFull, r[i].y, m);
-            d += imconj(r[i], xo);
-            x[i] = unrot(x[i], xo, cs);
-            r[i] = unrot(r[i], ro, cs);
+        for (int h = 0; h < NP; ++h) {
+            const float2 t = halves(imconj(r[h], swap(x[h])));
+            d += t.x + t.y;
         }
-        dfl_add(acc, d);
+    } else {
+        float up[NP / 2];
+        int n = 0;
+#pragma unroll
+        for (int h = 0; h < NP; ++h) {
+            if (h & (1 << q)) continue;
+            const int j = h | (1 << q);
+            const float2 t = halves(add2(imconj(r[h], x[j]), imconj(r[j], x[h])));
+            d += t.x;
+            up[n++] = t.y;
+        }
+#pragma unroll
+        for (int k = 0; k < NP / 2; ++k) d += up[k];
     }
+    return d;
 }
 
-// Sum of Im<r|X_q|x> over every register and lane qubit (only qubits 0 and 1
-// unless `all`), states unchanged; one qubit's terms at a time into the
-// compensated sum.
-template <int NR>
-__device__ __forceinline__ Dfl xterms(const float2 (&x)[NR], const float2 (&r)[NR], bool all) {
-    Dfl acc{0.f, 0.f};
+// The same over a lane qubit, given the partner's x.
+template <int NP>
+__device__ __forceinline__ float xterm_lane(const C2 (&xo)[NP], const C2 (&r)[NP]) {
+    float d = 0.f, up[NP];
 #pragma unroll
-    for (int rb = 0; (1 << rb) < NR; ++rb) {
-        if (!all && rb >= 2) continue;
-        float d = 0.f;
-#pragma unroll
-        for (int i = 0; i < NR; ++i) {
-            if (i & (1 << rb)) continue;
-            const int i2 = i | (1 << rb);
-            d += imconj(r[i], x[i2]) + imconj(r[i2], x[i]);
-        }
-        dfl_add(acc, d);
+    for (int h = 0; h < NP; ++h) {
+        const float2 t = halves(imconj(r[h], xo[h]));
+        d += t.x;
+        up[h] = t.y;
     }
-    if (!all) return acc;
 #pragma unroll
-    for (int lb = 0; lb < 5; ++lb) {
-        float d = 0.f;
-#pragma unroll
-        for (int i = 0; i < NR; ++i) {
-            float2 xo;
-            xo.x = __shfl_xor_sync(kFull, x[i].x, 1 << lb);
-            xo.y = __shfl_xor_sync(kFull, x[i].y, 1 << lb);
-            d += imconj(r[i], xo);
-        }
-        dfl_add(acc, d);
-    }
-    return acc;
+    for (int h = 0; h < NP; ++h) d += up[h];
+    return d;
 }
 
 // <Z_0 Z_1> sign of register i (qubits 0 and 1 are register bits 0 and 1).
 __host__ __device__ constexpr float zz_sign(int i) { return ((i ^ (i >> 1)) & 1) ? -1.f : 1.f; }
 
-#ifndef QAOA_SPLIT_GRAD_BLOCKS
-#define QAOA_SPLIT_GRAD_BLOCKS 4  // resident CTAs per SM of the adjoint core kernel
-#endif
+__device__ __forceinline__ float lds1(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void opaque(uint32_t &v) { asm volatile("" : "+r"(v)); }
 
+// Resident CTAs per SM.  Adjoint: 3 (168 registers, no spills; 2, 4 and 5:
+// 16.4, 17.4 and 18.8 against 15.8 ms on four cubic graphs n = 24, p = 3, 25
+// points); energy: 4 (128 registers; 2, 3 and 5: 10.0, 9.2 and 9.4 against 9.0
+// ms on the 6x6 torus).
+constexpr int kCoreGradBlocks = 3, kCoreEnergyBlocks = 4;
+
+// Rows of a warp's phase tables: 68 real parts, then 68 imaginary parts (a cone
+// has at most 64 cut bits); count bytes hold 2 c.
+constexpr int kCoreRow = 544, kCoreIm = 272;
+constexpr float kCoreScale = 2.f;
+inline size_t core_smem_bytes(int p, bool grad) { return size_t(4) * (p * kCoreRow + (grad ? 2 * p * 32 * sizeof(float2) : 0)); }
+
+// A warp takes L.tpw consecutive tiles of one item: the item's decoding, its
+// phase tables (staged in shared memory, rows of real parts and of imaginary
+// parts) and the warp reductions and atomics of the sums are per item and not
+// per tile.  The derivative sums gather per lane in compensated pairs in shared
+// memory meanwhile.
+//
+// Bound: instruction fetch and latency (ncu, adjoint, p = 3: 49% of the issue
+// slots, FP32 pipe 52%, no-instruction the first stall; 5,000 instructions of
+// straight-line code), the energy by shuffles and shared memory (55%).  Measured
+// against the unpacked kernel with one tile per task: four cubic graphs n = 24,
+// p = 3, 25 points, gradient 21.6 -> 15.8 ms; 6x6 torus, p = 3, 32 points, energy
+// 10.1 -> 8.8 ms (both with their outer passes).
 template <bool GRAD, int RB>
-__global__ void __launch_bounds__(128, GRAD ? QAOA_SPLIT_GRAD_BLOCKS : 3) split_core_kernel(const __grid_constant__ BigLaunch L) {
-    constexpr int NR = 1 << RB;
+__global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlocks) split_core_kernel(const __grid_constant__ BigLaunch L) {
+    constexpr int NR = 1 << RB, NP = NR / 2;
     constexpr int T = RB + 5;
     constexpr int NW = NR / 4;  // packed cut counts, 4 registers per word
-    const int lane = threadIdx.x & 31;
-    const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp_index();
-    const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
+    extern __shared__ __align__(256) unsigned char s_core[];
+    const int lane = threadIdx.x & 31, warp = warp_index();
+    const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp;
+    const int64_t nw = int64_t(gridDim.x) * (blockDim.x >> 5);
     const int nin = L.n_in;
     const int p = L.p;
-    const int64_t tiles = int64_t(1) << (nin - T);
-    const int64_t ntask = L.n_items * tiles;
+    const int tpw = L.tpw;
+    const int64_t per_item = (int64_t(1) << (nin - T)) / tpw;
+    const int64_t ntask = L.n_items * per_item;
     const int64_t block_amps = int64_t(1) << nin;
+    unsigned char *tab = s_core + warp * (p * kCoreRow);
+    float2 *sums = reinterpret_cast<float2 *>(s_core + (blockDim.x >> 5) * (p * kCoreRow)) + warp * (2 * p * 32) + lane;
+    const uint32_t tab0 = smem_addr(tab);
     for (int64_t task = gw; task < ntask; task += nw) {
-        const int64_t it = task / tiles;
-        const int64_t u = task - it * tiles;
+        const int64_t it = task / per_item;
+        const int64_t u0 = (task - it * per_item) * tpw;
         int ci;
         int64_t j, y;
         decode_item(L, L.item0 + it, ci, j, y);
         const DevCone *__restrict__ C = L.cones + L.cone_ids[ci];
-        if (C->n_in != nin) {
+        if (__any_sync(kFull, C->n_in != nin)) {
             if (lane == 0) atomicOr(L.status, 1);
             continue;
         }
         const int64_t gj = int64_t(C->graph) * L.P + j;
-        const float2 *__restrict__ lut = L.lut + gj * p * L.cmax1;
         const float4 *__restrict__ cs = L.cs + gj * p;
-        // cut word of the tile's fixed bits: shell block, outer qubits, lane qubits
+        __syncwarp();
+        {
+            const float2 *__restrict__ lut = L.lut + gj * p * L.cmax1;
+            for (int l = 0; l < p; ++l)
+                for (int e = lane; e < L.cmax1; e += 32) {
+                    const float2 v = __ldg(lut + l * L.cmax1 + e);
+                    *reinterpret_cast<float *>(tab + l * kCoreRow + 4 * e) = v.x;
+                    *reinterpret_cast<float *>(tab + l * kCoreRow + kCoreIm + 4 * e) = v.y;
+                }
+            if (GRAD)
+                for (int c = 0; c < 2 * p; ++c) sums[32 * c] = make_float2(0.f, 0.f);
+        }
+        __syncwarp();
+        // cut word of the item's fixed bits: shell block, lane qubits
         float mult = 1.f;
         uint64_t base = shell_block(C, L.shell, uint32_t(y), mult);
-        for (int q = T; q < nin; ++q)
-            if ((u >> (q - T)) & 1) base ^= C->col[q];
 #pragma unroll
         for (int lb = 0; lb < 5; ++lb)
             if ((lane >> lb) & 1) base ^= C->col[RB + lb];
-        // cut value of every register, one byte each (a cone has < 256 edges)
-        uint32_t cnt[NW];
-        {
-            const uint64_t c0 = C->col[0], c1 = C->col[1];
-            const uint64_t lo[4] = {0ull, c0, c1, c0 ^ c1};
-#pragma unroll
-            for (int w = 0; w < NW; ++w) {
-                uint64_t h = base;
-#pragma unroll
-                for (int t = 0; t < RB - 2; ++t)
-                    if ((w >> t) & 1) h ^= C->col[2 + t];
-                uint32_t packed = 0;
-#pragma unroll
-                for (int a = 0; a < 4; ++a) packed |= uint32_t(__popcll(lo[a] ^ h)) << (8 * a);
-                cnt[w] = packed;
-            }
-        }
-        auto cut = [&](int i) -> int { return int((cnt[i >> 2] >> (8 * (i & 3))) & 0xffu); };
-        float2 *__restrict__ sp = L.psi + it * block_amps + (u << T) + lane;
-        float2 x[NR];
-        if (L.load) {
-#pragma unroll
-            for (int i = 0; i < NR; ++i) x[i] = sp[i << 5];
-        } else {
-#pragma unroll
-            for (int i = 0; i < NR; ++i) x[i] = __ldg(lut + cut(i));
-        }
         const FirstMix f1 = first_mix(L, gj, nin);
-        // |psi|^2 = 2^-n kappa_1^(2 n_in) |x|^2 (the first mixer's factored form)
-        float sig = __int_as_float((127 - C->n) << 23) * f1.k2n;
-        // first mixer on the core qubits
-        first_mix_regs<NR, false>(x, 0, RB, f1);
-        first_mix_lanes<NR, false>(x, 5, f1);
-        for (int l = 1; l < p; ++l) {
-            const float2 *__restrict__ lt = lut + l * L.cmax1;
+        const float wgt = float(C->weight);
+        const float sig0 = __int_as_float((127 - C->n) << 23) * f1.k2n;
+        // In d/d gamma_l, C may be replaced by C - c0: Im<lambda|psi> =
+        // <psi_end|O|psi_end> is zero within every core tile, and c0 = m/2
+        // (the mean cut value) removes most of the cancellation in the FP32
+        // sums.  Counts are bytes of kCoreScale c; 2^23 + kCoreScale c0 here.
+        const float b0 = 8388608.f + 0.5f * kCoreScale * float(C->m);
+        auto add_sum = [&](int c, Dfl v) {
+            const float2 s = sums[32 * c];
+            Dfl a{s.x, s.y};
+            dfl_add(a, v);
+            sums[32 * c] = make_float2(a.hi, a.lo);
+        };
+        Dfl e_sum{0.f, 0.f}, t_sum{0.f, 0.f};  // of the warp's tile sums
+        for (int64_t u = u0; u < u0 + tpw; ++u) {
+            uint64_t tb = base;
+            for (int q = T; q < nin; ++q)
+                if ((u >> (q - T)) & 1) tb ^= C->col[q];
+            // cut value of every register, one byte each, times kCoreScale (a cone has at most 64 cut bits)
+            uint32_t cnt[NW];
+            {
+                const uint64_t c0 = C->col[0], c1 = C->col[1];
+                const uint64_t lo[4] = {0ull, c0, c1, c0 ^ c1};
 #pragma unroll
-            for (int i = 0; i < NR; ++i) x[i] = cmul(x[i], __ldg(lt + cut(i)));
-            const int kl = C->k[l];
-            if (GRAD) {  // the adjoint keeps exact rotations (its derivative terms need them)
-                const float4 c_s = __ldg(cs + l);
-                mix_regs<NR>(x, kl < RB ? kl : RB, c_s);
-                if (kl > RB) mix_lanes<NR>(x, kl - RB, c_s);
-            } else {  // the energy: the factored form, two FMAs per output, kappa^(2 k_l) into sigma
-                const FirstMix fl = layer_mix(L, gj, l, kl);
-                first_mix_regs<NR, false>(x, 0, kl < RB ? kl : RB, fl);
-                if (kl > RB) first_mix_lanes<NR, false>(x, kl - RB, fl);
-                sig *= fl.k2n;
+                for (int w = 0; w < NW; ++w) {
+                    uint64_t h = tb;
+#pragma unroll
+                    for (int t = 0; t < RB - 2; ++t)
+                        if ((w >> t) & 1) h ^= C->col[2 + t];
+                    uint32_t packed = 0;
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) packed |= uint32_t(__popcll(lo[a] ^ h)) << (8 * a);
+                    cnt[w] = packed * uint32_t(kCoreScale);
+                }
+            }
+            // table entries of registers h and h + NP in the row of layer l
+            auto entry = [&](int h, int l) -> C2 {
+                const uint32_t row = tab0 + l * kCoreRow;
+                const uint32_t a = row + (__byte_perm(cnt[h >> 2], 0u, 0x4440u | uint32_t(h & 3)) << 1);
+                const uint32_t b = row + (__byte_perm(cnt[(h >> 2) + NW / 2], 0u, 0x4440u | uint32_t(h & 3)) << 1);
+                return C2{p2(lds1(a), lds1(b)), p2(lds1(a + kCoreIm), lds1(b + kCoreIm))};
+            };
+            auto weight = [&](int h) -> P2 {  // kCoreScale (c - c0)
+                return add2(p2(__uint_as_float(__byte_perm(cnt[h >> 2], 0x4B000000u, 0x7540u | uint32_t(h & 3))),
+                               __uint_as_float(
+                                   __byte_perm(cnt[(h >> 2) + NW / 2], 0x4B000000u, 0x7540u | uint32_t(h & 3)))),
+                            splat(-b0));
+            };
+            float2 *__restrict__ sp = L.psi + it * block_amps + (u << T) + lane;
+            C2 x[NP];
+            if (L.load) {
+#pragma unroll
+                for (int h = 0; h < NP; ++h) {
+                    const float2 v = sp[h << 5], w = sp[(h + NP) << 5];
+                    x[h] = C2{p2(v.x, w.x), p2(v.y, w.y)};
+                }
+            } else {
+#pragma unroll
+                for (int h = 0; h < NP; ++h) x[h] = entry(h, 0);
+            }
+            // |psi|^2 = 2^-n kappa_1^(2 n_in) |x|^2 (the first mixer's factored form)
+            float sig = sig0;
+            // first mixer on the core qubits
+            first_mix2<NP, false, GRAD>(x, RB, 5, f1);
+            for (int l = 1; l < p; ++l) {
+#pragma unroll
+                for (int w = 0; w < NW; ++w) opaque(cnt[w]);
+#pragma unroll
+                for (int h = 0; h < NP; ++h) x[h] = cmul_ri(x[h], entry(h, l));
+                const int kl = uniform(C->k[l]);
+                if (GRAD) {  // the adjoint keeps exact rotations (its derivative terms need them)
+                    const float4 c_s = __ldg(cs + l);
+                    on_qubits<NP>(x, kl, kl - RB, [&](const C2 &a, const C2 &b) { return rot2<false>(a, b, c_s); });
+                } else {  // the energy: the factored form, two FMAs per output, kappa^(2 k_l) into sigma
+                    const FirstMix fl = layer_mix(L, gj, l, kl);
+                    first_mix2<NP, false, false>(x, kl, kl - RB, fl);
+                    sig *= fl.k2n;
+                }
+            }
+            float acc = 0.f;
+            {
+                float up[NP];
+                const bool norm = !GRAD && L.norm;
+#pragma unroll
+                for (int h = 0; h < NP; ++h) {
+                    const float2 v = halves(fma2(x[h].r, x[h].r, mul2(x[h].i, x[h].i)));
+                    const float s = norm ? 1.f : zz_sign(h);
+                    acc = fmaf(s, v.x, acc);
+                    up[h] = s * v.y;  // registers h and h + NP have the same sign
+                }
+#pragma unroll
+                for (int h = 0; h < NP; ++h) acc += up[h];
+            }
+            {
+                const float tv = acc * sig * mult;  // this tile's share of <Z_0 Z_1>
+                dfl_add(e_sum, warp_sum(-0.5f * wgt * tv));
+                if (L.terms) dfl_add(t_sum, warp_sum(tv));
+            }
+            if (GRAD) {
+                C2 r[NP];
+#pragma unroll
+                for (int h = 0; h < NP; ++h) {
+                    const P2 s = splat(-0.5f * zz_sign(h));
+                    r[h] = C2{mul2(s, x[h].r), mul2(s, x[h].i)};
+                }
+                for (int l = p - 1; l >= 1; --l) {
+                    const float4 c_s = __ldg(cs + l);
+                    const int kl = uniform(C->k[l]);
+                    auto un = [&](const C2 &a, const C2 &b) { return rot2<true>(a, b, c_s); };
+                    Dfl d{0.f, 0.f};
+#pragma unroll
+                    for (int q = 0; q < RB; ++q) {
+                        if (q < kl) {
+                            dfl_add(d, xterm_reg<NP>(x, r, q));
+                            on_reg<NP>(x, q, un);
+                            on_reg<NP>(r, q, un);
+                        }
+                    }
+#pragma unroll 1
+                    for (int lb = 0; lb < kl - RB; ++lb) {
+                        C2 xo[NP];
+#pragma unroll
+                        for (int h = 0; h < NP; ++h) xo[h] = shfl_xor(x[h], 1 << lb);
+                        dfl_add(d, xterm_lane<NP>(xo, r));
+#pragma unroll
+                        for (int h = 0; h < NP; ++h) {
+                            x[h] = un(x[h], xo[h]);
+                            r[h] = un(r[h], shfl_xor(r[h], 1 << lb));
+                        }
+                    }
+                    add_sum(p + l, d);
+#pragma unroll
+                    for (int w = 0; w < NW; ++w) opaque(cnt[w]);
+                    float dg = 0.f, uw[NP], uv[NP];
+#pragma unroll
+                    for (int h = 0; h < NP; ++h) {
+                        const float2 w = halves(weight(h)), v = halves(imconj(r[h], x[h]));
+                        dg = fmaf(w.x, v.x, dg);
+                        uw[h] = w.y;
+                        uv[h] = v.y;
+                        const C2 ph = entry(h, l);
+                        x[h] = cmulc(x[h], ph);
+                        r[h] = cmulc(r[h], ph);
+                    }
+#pragma unroll
+                    for (int h = 0; h < NP; ++h) dg = fmaf(uw[h], uv[h], dg);
+                    add_sum(l, Dfl{dg * (1.f / kCoreScale), 0.f});
+                }
+                // first mixer: the core qubits' terms, then lambda alone un-mixed
+                // At p = 1 the first layer is the last: lambda = O psi with
+                // O = -1/2 Z_0 Z_1, and <psi|O X_q|psi> is real for every q other
+                // than 0 and 1 (X_q and O commute), so only those two contribute.
+                {
+                    Dfl d{0.f, 0.f};
+#pragma unroll
+                    for (int q = 0; q < RB; ++q)
+                        if (q < 2 || p > 1) dfl_add(d, xterm_reg<NP>(x, r, q));
+                    if (p > 1) {
+#pragma unroll 1
+                        for (int lb = 0; lb < 5; ++lb) {
+                            C2 xo[NP];
+#pragma unroll
+                            for (int h = 0; h < NP; ++h) xo[h] = shfl_xor(x[h], 1 << lb);
+                            dfl_add(d, xterm_lane<NP>(xo, r));
+                        }
+                    }
+                    add_sum(p, d);
+                }
+                first_mix2<NP, true, true>(r, RB, 5, f1);
+#pragma unroll
+                for (int h = 0; h < NP; ++h) {
+                    const float2 a = halves(r[h].r), b = halves(r[h].i);
+                    sp[h << 5] = make_float2(a.x, b.x);
+                    sp[(h + NP) << 5] = make_float2(a.y, b.y);
+                }
             }
         }
-        float acc = 0.f;
-#pragma unroll
-        for (int i = 0; i < NR; ++i) acc += (GRAD || !L.norm ? zz_sign(i) : 1.f) * fmaf(x[i].x, x[i].x, x[i].y * x[i].y);
-        const float tv = acc * sig * mult;  // this tile's share of <Z_0 Z_1>
-        add_gp(-0.5f * float(C->weight) * tv, L.energy, gj);
-        if (L.terms) add_gp(tv, L.terms, C->rep * L.P + j);
+        if (lane == 0) {
+            atomicAdd(L.energy + gj, dfl_value(e_sum));
+            if (L.terms) atomicAdd(L.terms + C->rep * L.P + j, dfl_value(t_sum));
+        }
         if (GRAD) {
-            const float wgt2 = 2.f * float(C->weight) * mult * sig;
-            float2 r[NR];
-#pragma unroll
-            for (int i = 0; i < NR; ++i) {
-                const float h = -0.5f * zz_sign(i);
-                r[i] = make_float2(h * x[i].x, h * x[i].y);
+            const float wgt2 = 2.f * wgt * mult * sig0;
+            for (int l = 1; l < p; ++l) {
+                add_gp(Dfl{sums[32 * (p + l)].x, sums[32 * (p + l)].y}, wgt2, L.grad, gj * 2 * p + p + l);
+                add_gp(Dfl{sums[32 * l].x, sums[32 * l].y}, wgt2, L.grad, gj * 2 * p + l);
             }
-            // In d/d gamma_l, C may be replaced by C - c0: Im<lambda|psi> =
-            // <psi_end|O|psi_end> is zero within every core tile, and c0 = m/2
-            // (the mean cut value) removes most of the cancellation in the
-            // FP32 sums.
-            const float c0 = 0.5f * float(C->m);
-            for (int l = p - 1; l >= 1; --l) {
-                const float4 c_s = __ldg(cs + l);
-                const int kl = C->k[l];
-                Dfl d{0.f, 0.f};
-                unmix_regs_d<NR>(x, r, kl < RB ? kl : RB, c_s, d);
-                if (kl > RB) unmix_lanes_d<NR>(x, r, kl - RB, c_s, d);
-                add_gp(d, wgt2, L.grad, gj * 2 * p + p + l);
-                const float2 *__restrict__ lt = lut + l * L.cmax1;
-                // keep the shifted cut values from being hoisted out of the layer
-                // loop into sixteen live registers
-#pragma unroll
-                for (int w = 0; w < NW; ++w) asm volatile("" : "+r"(cnt[w]));
-                float dg = 0.f;
-#pragma unroll
-                for (int i = 0; i < NR; ++i) {
-                    const int c = cut(i);
-                    dg = fmaf(float(c) - c0, imconj(r[i], x[i]), dg);
-                    const float2 ph = __ldg(lt + c);
-                    x[i] = cmulc(x[i], ph);
-                    r[i] = cmulc(r[i], ph);
-                }
-                add_gp(Dfl{dg, 0.f}, wgt2, L.grad, gj * 2 * p + l);
-            }
-            // first mixer: the core qubits' terms, then lambda alone un-mixed
-            // At p = 1 the first layer is the last: lambda = O psi with
-            // O = -1/2 Z_0 Z_1, and <psi|O X_q|psi> is real for every q other
-            // than 0 and 1 (X_q and O commute), so only those two contribute.
-            add_gp(xterms<NR>(x, r, p > 1), wgt2, L.grad, gj * 2 * p + p);
-            first_mix_regs<NR, true>(r, 0, RB, f1);
-            first_mix_lanes<NR, true>(r, 5, f1);
-#pragma unroll
-            for (int i = 0; i < NR; ++i) sp[i << 5] = r[i];
+            add_gp(Dfl{sums[32 * p].x, sums[32 * p].y}, wgt2, L.grad, gj * 2 * p + p);
         }
     }
 }
@@ -554,8 +684,6 @@ __device__ __forceinline__ int swz(int s) { return s ^ ((__popc(s >> 4) & 1) << 
 __device__ __forceinline__ int sidx(int s, bool swizzled) { return swizzled ? swz(s) : s; }
 
 // ---- tensor-memory-accelerator helpers (one thread issues, an mbarrier tracks loads)
-__device__ __forceinline__ uint32_t smem_addr(const void *p) { return uint32_t(__cvta_generic_to_shared(p)); }
-
 __device__ __forceinline__ void mbar_init(uint64_t *bar) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -893,7 +1021,7 @@ cudaError_t split_prepare() {
 cudaError_t launch_split_wave(BigLaunch B, bool grad, int chunk_window, int64_t &launches, cudaStream_t s) {
     const int cw_max = chunk_window < 6 ? 6 : (chunk_window > kChunkMaxW ? kChunkMaxW : chunk_window);
     const int RB = grad ? kSplitRbGrad : kSplitRbEnergy, T = RB + 5;
-    const int nin = B.n_in;
+    const int nin = B.n_in, p = B.p;
     B.rb = RB;
     // Outer qubit windows: shared-memory chunks of up to kChunkMaxW qubits
     // while more than five remain, then one register window of at most five.
@@ -957,14 +1085,21 @@ cudaError_t launch_split_wave(BigLaunch B, bool grad, int chunk_window, int64_t 
     for (size_t w = 0; w < win.size() && e == cudaSuccess; ++w) e = outer(w == 0 ? kOuterGen : kOuterMix, w, 1);
     if (e != cudaSuccess) return e;
     B.load = win.empty() ? 0 : 1;
-    const int64_t core_tasks = B.n_items << (nin - T);
-    if (grad) {
-        const void *fn = (const void *)split_core_kernel<true, kSplitRbGrad>;
-        split_core_kernel<true, kSplitRbGrad><<<grid_for(fn, core_tasks), 128, 0, s>>>(B);
-    } else {
-        const void *fn = (const void *)split_core_kernel<false, kSplitRbEnergy>;
-        split_core_kernel<false, kSplitRbEnergy><<<grid_for(fn, core_tasks), 128, 0, s>>>(B);
-    }
+    // tiles per warp task: as many as leave two tasks for every resident warp (of 1, 2, 4, 8, 16: 9.46, 8.77, 8.94,
+    // 9.02, 9.37 ms on the 6x6 torus at p = 3, energy, 32 points; within 3% for four cubic graphs n = 24, gradient)
+    const void *core = grad ? (const void *)split_core_kernel<true, kSplitRbGrad>
+                            : (const void *)split_core_kernel<false, kSplitRbEnergy>;
+    const size_t core_smem = core_smem_bytes(p, grad);
+    const int core_grid = occupancy_grid(core, 128, core_smem);
+    B.tpw = 1;
+    while (B.tpw < (1 << std::min(nin - T, 6)) && (B.n_items << (nin - T)) / (2 * B.tpw) >= int64_t(core_grid) * 4 * 2)
+        B.tpw *= 2;
+    const int64_t core_tasks = (B.n_items << (nin - T)) / B.tpw;
+    const int grid = int(std::min<int64_t>(core_grid, std::max<int64_t>(1, (core_tasks + 3) / 4)));
+    if (grad)
+        split_core_kernel<true, kSplitRbGrad><<<grid, 128, core_smem, s>>>(B);
+    else
+        split_core_kernel<false, kSplitRbEnergy><<<grid, 128, core_smem, s>>>(B);
     ++launches;
     if ((e = cudaGetLastError()) != cudaSuccess || !grad) return e;
     for (size_t w = win.size(); w-- > 1 && e == cudaSuccess;) e = outer(kOuterMix, w, -1);

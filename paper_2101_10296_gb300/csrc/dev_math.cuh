@@ -16,6 +16,10 @@ constexpr unsigned kFull = 0xffffffffu;
 // 30-vertex circulant at p = 4: 2.15 -> 1.81 ms).
 __device__ __forceinline__ int warp_index() { return __shfl_sync(kFull, int(threadIdx.x >> 5), 0); }
 
+// A value every lane holds alike (loaded from one address, say), told to the
+// compiler the same way.
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(kFull, v, 0); }
+
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }

@@ -58,9 +58,14 @@ struct C2 {
 };
 
 // a b, a conj(b) and Im(conj(a) b); which product is rounded by itself follows
-// what the compiler makes of cmul, cmulc and imconj (dev_math.cuh)
+// what the compiler made of cmul, cmulc and imconj (dev_math.cuh) in the scalar
+// kernels: the imaginary part of a product had a.i b.r in the FMA in the
+// register kernel (cmul) and a.r b.i in the large-state kernels (cmul_ri)
 __device__ __forceinline__ C2 cmul(const C2 &a, const C2 &b) {
     return C2{fma2(a.r, b.r, neg(mul2(a.i, b.i))), fma2(a.i, b.r, mul2(a.r, b.i))};
+}
+__device__ __forceinline__ C2 cmul_ri(const C2 &a, const C2 &b) {
+    return C2{fma2(a.r, b.r, neg(mul2(a.i, b.i))), fma2(a.r, b.i, mul2(a.i, b.r))};
 }
 __device__ __forceinline__ C2 cmulc(const C2 &a, const C2 &b) {
     return C2{fma2(a.r, b.r, mul2(a.i, b.i)), fma2(a.i, b.r, neg(mul2(a.r, b.i)))};
