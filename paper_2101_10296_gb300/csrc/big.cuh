@@ -72,7 +72,7 @@ struct BigLaunch {
     int32_t x0, x1;           // kOuterFirst: outer qubits [x0, x1) outside the window
     int32_t mode, sign;       // SplitOuterMode; +1 mix, -1 un-mix (kOuterMix)
     int32_t load;             // core pass: load the tile (1) or generate layer 1's phase state (0)
-    int32_t tpw;              // core pass: consecutive tiles of an item per warp task (a power of two)
+    int32_t tpw;              // consecutive tiles of an item per warp task (a power of two)
 };
 
 // Cones of one shape share n_in and k; items of a wave are numbered cone by

@@ -60,21 +60,24 @@ namespace {
 // Hessian times that shift -- as large as the whole 1e-4 tolerance at points
 // where |grad E| ~ 1e-3 |E|.  The adjoint's passes use it; the energy's need
 // not (E moves by grad E . delta beta).
+//
+// Here on one amplitude, its real and imaginary parts a packed pair: the partner
+// enters with the halves exchanged.
 template <bool B, bool INV, bool LO>
-__device__ __forceinline__ float2 fmix(float2 me, float2 o, float a, float alo) {
+__device__ __forceinline__ P2 fmix(P2 me, P2 o, float a, float alo) {
+    const P2 so = swap(o);
     if (!B) {
-        const float ox = LO ? fmaf(INV ? -alo : alo, o.y, me.x) : me.x;
-        const float oy = LO ? fmaf(INV ? alo : -alo, o.x, me.y) : me.y;
-        return INV ? make_float2(fmaf(-a, o.y, ox), fmaf(a, o.x, oy)) : make_float2(fmaf(a, o.y, ox), fmaf(-a, o.x, oy));
+        const P2 ox = LO ? fma2(INV ? p2(-alo, alo) : p2(alo, -alo), so, me) : me;
+        return fma2(INV ? p2(-a, a) : p2(a, -a), so, ox);
     }
-    const float px = LO ? fmaf(alo, me.x, INV ? -o.y : o.y) : (INV ? -o.y : o.y);
-    const float py = LO ? fmaf(alo, me.y, INV ? o.x : -o.x) : (INV ? o.x : -o.x);
-    return make_float2(fmaf(a, me.x, px), fmaf(a, me.y, py));
+    const float2 h = halves(so);
+    const P2 io = INV ? p2(-h.x, h.y) : p2(h.x, -h.y);  // i o, or -i o
+    return fma2(splat(a), me, LO ? fma2(splat(alo), me, io) : io);
 }
 
 // D (or D') on register bits [r0, r1).
 template <int NR, bool B, bool INV, bool LO>
-__device__ __forceinline__ void fmix_regs(float2 (&x)[NR], int r0, int r1, float a, float alo) {
+__device__ __forceinline__ void fmix_regs(P2 (&x)[NR], int r0, int r1, float a, float alo) {
 #pragma unroll
     for (int rb = 0; (1 << rb) < NR; ++rb) {
         if (rb >= r0 && rb < r1) {
@@ -82,25 +85,10 @@ __device__ __forceinline__ void fmix_regs(float2 (&x)[NR], int r0, int r1, float
             for (int i = 0; i < NR; ++i) {
                 if (i & (1 << rb)) continue;
                 const int i2 = i | (1 << rb);
-                const float2 u = x[i], v = x[i2];
+                const P2 u = x[i], v = x[i2];
                 x[i] = fmix<B, INV, LO>(u, v, a, alo);
                 x[i2] = fmix<B, INV, LO>(v, u, a, alo);
             }
-        }
-    }
-}
-
-// D (or D') on lane bits [0, nb).
-template <int NR, bool B, bool INV, bool LO>
-__device__ __forceinline__ void fmix_lanes(float2 (&x)[NR], int nb, float a, float alo) {
-    for (int lb = 0; lb < nb; ++lb) {
-        const int m = 1 << lb;
-#pragma unroll
-        for (int i = 0; i < NR; ++i) {
-            float2 o;
-            o.x = __shfl_xor_sync(kFull, x[i].x, m);
-            o.y = __shfl_xor_sync(kFull, x[i].y, m);
-            x[i] = fmix<B, INV, LO>(x[i], o, a, alo);
         }
     }
 }
@@ -133,33 +121,28 @@ __device__ __forceinline__ FirstMix layer_mix(const BigLaunch &L, int64_t gj, in
     return f;
 }
 
-template <int NR, bool INV>
-__device__ __forceinline__ void first_mix_regs(float2 (&x)[NR], int r0, int r1, const FirstMix &f) {
-    if (f.alo != 0.f) {
-        if (f.b)
-            fmix_regs<NR, true, INV, true>(x, r0, r1, f.a, f.alo);
-        else
-            fmix_regs<NR, false, INV, true>(x, r0, r1, f.a, f.alo);
-    } else if (f.b) {
-        fmix_regs<NR, true, INV, false>(x, r0, r1, f.a, 0.f);
-    } else {
-        fmix_regs<NR, false, INV, false>(x, r0, r1, f.a, 0.f);
-    }
+template <int NR, bool INV, bool LO>
+__device__ __forceinline__ void first_mix_regs(P2 (&x)[NR], int r0, int r1, const FirstMix &f) {
+    if (f.b)
+        fmix_regs<NR, true, INV, LO>(x, r0, r1, f.a, f.alo);
+    else
+        fmix_regs<NR, false, INV, LO>(x, r0, r1, f.a, f.alo);
 }
 
-template <int NR, bool INV>
-__device__ __forceinline__ void first_mix_lanes(float2 (&x)[NR], int nb, const FirstMix &f) {
-    if (f.alo != 0.f) {
-        if (f.b)
-            fmix_lanes<NR, true, INV, true>(x, nb, f.a, f.alo);
-        else
-            fmix_lanes<NR, false, INV, true>(x, nb, f.a, f.alo);
-    } else if (f.b) {
-        fmix_lanes<NR, true, INV, false>(x, nb, f.a, 0.f);
-    } else {
-        fmix_lanes<NR, false, INV, false>(x, nb, f.a, 0.f);
-    }
+// An amplitude as a packed pair.
+__device__ __forceinline__ P2 load_amp(const float2 *p) { return P2{*reinterpret_cast<const unsigned long long *>(p)}; }
+__device__ __forceinline__ void store_amp(float2 *p, P2 v) { *reinterpret_cast<unsigned long long *>(p) = v.v; }
+
+// Cut words as 32 bits where every cone of the plan fits them, else 64.
+__device__ __forceinline__ int popc_w(uint32_t x) { return __popc(x); }
+__device__ __forceinline__ int popc_w(uint64_t x) { return __popcll(x); }
+// XOR over the lanes.
+__device__ __forceinline__ uint32_t warp_xor(uint32_t x) { return __reduce_xor_sync(kFull, x); }
+__device__ __forceinline__ uint64_t warp_xor(uint64_t x) {
+    return (uint64_t(__reduce_xor_sync(kFull, uint32_t(x >> 32))) << 32) | __reduce_xor_sync(kFull, uint32_t(x));
 }
+// c - c0 of a cut value, given b0 = 2^22 + c0 (halves are exact at that size)
+__device__ __forceinline__ float cut_minus(int c, float b0) { return __uint_as_float(0x4A800000u + 2u * uint32_t(c)) - b0; }
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return uint32_t(__cvta_generic_to_shared(p)); }
 
@@ -548,111 +531,194 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
     }
 }
 
+// ---------------------------------------------------------------- outer passes
+constexpr int kOuterRow = 68;  // table entries: a cone has at most 64 cut bits
+template <bool V>
+struct BoolTag {
+    static constexpr bool value = V;
+};
+
 // Qubit held by storage address bit a (see the layout above).
 __device__ __forceinline__ int qubit_of(int a, int rb) { return a < 5 ? rb + a : (a < rb + 5 ? a - 5 : a); }
 
-template <int MODE>
+// A warp takes L.tpw consecutive tiles of an item (lanes = address bits 0..4,
+// registers = the window).  The item's first-layer table sits in shared memory,
+// a lane holds the cut word of one address bit outside the window (a tile's
+// fixed word is one XOR reduction), and the derivative sums gather over the
+// tiles.  The state is held an amplitude per packed pair; kOuterFirst, which
+// forms pair terms, holds registers h and h + 16 together as the core pass does.
+// Blocks per SM: 4 and 3 (generation at 3 and 5, the others at 2 and 4: no faster).
+// Generation was bound by the integer pipe (64-bit popcounts and table lookups in
+// global memory, 50%).  With the chunk passes changed alike, against scalar
+// registers and one tile per task: four cubic graphs n = 24, p = 3, 25 points,
+// gradient 15.8 -> 14.4 ms, energy 3.7 -> 3.3 ms; 6x6 torus, p = 3, 32 points,
+// energy 8.8 -> 8.3 ms; Q_12 full cone, 32 points, energy 4.5 -> 4.15 ms.
+template <int MODE, bool LO, typename MT>
 __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_kernel(const __grid_constant__ BigLaunch L) {
-    const int lane = threadIdx.x & 31;
-    const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp_index();
-    const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
+    __shared__ __align__(16) float s_tab[4][MODE == kOuterMix ? 4 : 2 * kOuterRow];
+    const int lane = threadIdx.x & 31, warp = warp_index();
+    const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp;
+    const int64_t nw = int64_t(gridDim.x) * (blockDim.x >> 5);
     const int nin = L.n_in, b = L.b, RB = L.rb;
     const int r0 = L.w0 - b, r1 = L.w1 - b;  // register bits of the outer qubits to mix
     const int p = L.p;
-    const int64_t tiles = int64_t(1) << (nin - 10);
-    const int64_t ntask = L.n_items * tiles;
+    const int tpw = L.tpw;
+    const int64_t per_item = (int64_t(1) << (nin - 10)) / tpw;
+    const int64_t ntask = L.n_items * per_item;
     const int64_t block_amps = int64_t(1) << nin;
     const int64_t lowmask = (int64_t(1) << (b - 5)) - 1;
     for (int64_t task = gw; task < ntask; task += nw) {
-        const int64_t it = task / tiles;
-        const int64_t tile = task - it * tiles;
+        const int64_t it = task / per_item;
+        const int64_t tile0 = (task - it * per_item) * tpw;
         int ci;
         int64_t j, y;
         decode_item(L, L.item0 + it, ci, j, y);
         const DevCone *__restrict__ C = L.cones + L.cone_ids[ci];
-        if (C->n_in != nin) {
+        if (__any_sync(kFull, C->n_in != nin)) {
             if (lane == 0) atomicOr(L.status, 1);
             continue;
         }
         const int64_t gj = int64_t(C->graph) * L.P + j;
         const FirstMix f1 = first_mix(L, gj, nin);
-        // address of (lane, register i) = xb | (i << b) | lane
-        const int64_t xb = ((tile & lowmask) << 5) | ((tile >> (b - 5)) << (b + 5));
-        float2 *__restrict__ sp = L.psi + it * block_amps + xb + lane;
-        float2 x[32];
-        if (MODE != kOuterGen) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) x[i] = sp[int64_t(i) << b];
-        }
-        if (MODE == kOuterMix) {
-            if (L.sign > 0)
-                first_mix_regs<32, false>(x, r0, r1, f1);
-            else
-                first_mix_regs<32, true>(x, r0, r1, f1);
-        } else {
-            const float2 *__restrict__ lut = L.lut + gj * p * L.cmax1;  // first layer's phase table
-            float mult = 1.f;
-            uint64_t base = shell_block(C, L.shell, uint32_t(y), mult);
+        float mult = 1.f;
+        MT item_w = 0, bit_w = 0, lo[4], wh[8];
+        if (MODE != kOuterMix) {
+            // first layer's phase table: entries (kOuterGen), or real parts, then imaginary parts
+            __syncwarp();
+            const float2 *__restrict__ lut = L.lut + gj * p * L.cmax1;
+            for (int e = lane; e < L.cmax1; e += 32) {
+                const float2 v = __ldg(lut + e);
+                if (MODE == kOuterGen) {
+                    reinterpret_cast<float2 *>(s_tab[warp])[e] = v;
+                } else {
+                    s_tab[warp][e] = v.x;
+                    s_tab[warp][kOuterRow + e] = v.y;
+                }
+            }
+            __syncwarp();
+            item_w = MT(shell_block(C, L.shell, uint32_t(y), mult));
 #pragma unroll
             for (int lb = 0; lb < 5; ++lb)
-                if ((lane >> lb) & 1) base ^= C->col[RB + lb];
-            for (int a = 5; a < nin; ++a)
-                if ((a < b || a >= b + 5) && ((xb >> a) & 1)) base ^= C->col[qubit_of(a, RB)];
-            uint64_t lo[4], hi[8];
-            {
-                const uint64_t c0 = C->col[qubit_of(b, RB)], c1 = C->col[qubit_of(b + 1, RB)];
-                const uint64_t c2 = C->col[qubit_of(b + 2, RB)], c3 = C->col[qubit_of(b + 3, RB)];
-                const uint64_t c4 = C->col[qubit_of(b + 4, RB)];
-                lo[0] = 0;
-                lo[1] = c0;
-                lo[2] = c1;
-                lo[3] = c0 ^ c1;
+                if ((lane >> lb) & 1) item_w ^= MT(C->col[RB + lb]);
+            if (lane >= 5 && lane < nin && (lane < b || lane >= b + 5)) bit_w = MT(C->col[qubit_of(lane, RB)]);
+            const MT c0 = MT(C->col[qubit_of(b, RB)]), c1 = MT(C->col[qubit_of(b + 1, RB)]);
+            const MT c2 = MT(C->col[qubit_of(b + 2, RB)]), c3 = MT(C->col[qubit_of(b + 3, RB)]);
+            const MT c4 = MT(C->col[qubit_of(b + 4, RB)]);
+            lo[0] = 0;
+            lo[1] = c0;
+            lo[2] = c1;
+            lo[3] = c0 ^ c1;
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    hi[k] = base ^ ((k & 1) ? c2 : 0ull) ^ ((k & 2) ? c3 : 0ull) ^ ((k & 4) ? c4 : 0ull);
-            }
-            if (MODE == kOuterGen) {
+            for (int k = 0; k < 8; ++k) wh[k] = ((k & 1) ? c2 : MT(0)) ^ ((k & 2) ? c3 : MT(0)) ^ ((k & 4) ? c4 : MT(0));
+        }
+        Dfl s_dg{0.f, 0.f}, s_db{0.f, 0.f};
+        for (int64_t tile = tile0; tile < tile0 + tpw; ++tile) {
+            // address of (lane, register i) = xb | (i << b) | lane
+            const int64_t xb = ((tile & lowmask) << 5) | ((tile >> (b - 5)) << (b + 5));
+            float2 *__restrict__ sp = L.psi + it * block_amps + xb + lane;
+            MT base = 0;
+            if (MODE != kOuterMix) base = item_w ^ warp_xor(((xb >> lane) & 1) ? bit_w : MT(0));
+            if constexpr (MODE == kOuterFirst) {
+                C2 x[16];  // lambda
 #pragma unroll
-                for (int i = 0; i < 32; ++i) x[i] = __ldg(lut + __popcll(lo[i & 3] ^ hi[i >> 2]));
-                first_mix_regs<32, false>(x, r0, r1, f1);
-            } else {  // kOuterFirst: x holds lambda
-                first_mix_regs<32, true>(x, r0, r1, f1);
+                for (int h = 0; h < 16; ++h) {
+                    const float2 u = sp[int64_t(h) << b], v = sp[int64_t(h + 16) << b];
+                    x[h] = C2{p2(u.x, v.x), p2(u.y, v.y)};
+                }
+                auto unmix = [&](auto form) {
+#pragma unroll
+                    for (int q = 0; q < 5; ++q)
+                        if (q >= r0 && q < r1)
+                            on_reg<16>(x, q, [&](const C2 &u, const C2 &v) {
+                                return fmix2<decltype(form)::value, true, LO>(u, v, f1.a, f1.alo);
+                            });
+                };
+                if (f1.b)
+                    unmix(BoolTag<true>{});
+                else
+                    unmix(BoolTag<false>{});
                 // the outer qubits' mixer terms vanish at p = 1, where the first
                 // layer is the last (only qubits 0 and 1 contribute there)
                 const bool outer_terms = p > 1;
-                const float c0 = 0.5f * float(C->m);  // Im<lambda|psi> = 0: C - c0 in place of C
-                float dg = 0.f, dq[5] = {0.f, 0.f, 0.f, 0.f, 0.f};  // per window qubit
+                const float b0 = 4194304.f + 0.5f * float(C->m);  // Im<lambda|psi> = 0: C - c0 in place of C
+                const float *tr = s_tab[warp], *ti = s_tab[warp] + kOuterRow;
+                // state before the first mixer, times 2^(n/2), of registers h and h + 16
+                auto phase = [&](MT w, int h, int &cl, int &cu) -> C2 {
+                    cl = popc_w(MT(lo[h & 3] ^ wh[h >> 2] ^ w));
+                    cu = popc_w(MT(lo[h & 3] ^ wh[(h >> 2) + 4] ^ w));
+                    return C2{p2(tr[cl], tr[cu]), p2(ti[cl], ti[cu])};
+                };
+                C2 ph[16];
+                float dg = 0.f, uw[16], uv[16];
 #pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const int c = __popcll(lo[i & 3] ^ hi[i >> 2]);
-                    const float2 ph = __ldg(lut + c);  // state before the first mixer, times 2^(n/2)
-                    dg = fmaf(float(c) - c0, imconj(x[i], ph), dg);
-                    if (outer_terms) {
+                for (int h = 0; h < 16; ++h) {
+                    int cl, cu;
+                    ph[h] = phase(base, h, cl, cu);
+                    const float2 v = halves(imconj(x[h], ph[h]));
+                    dg = fmaf(cut_minus(cl, b0), v.x, dg);
+                    uw[h] = cut_minus(cu, b0);
+                    uv[h] = v.y;
+                }
 #pragma unroll
-                        for (int rb = 0; rb < 5; ++rb)
-                            if (rb >= r0 && rb < r1) dq[rb] += imconj(x[i ^ (1 << rb)], ph);
+                for (int h = 0; h < 16; ++h) dg = fmaf(uw[h], uv[h], dg);
+                dfl_add(s_dg, Dfl{dg, 0.f});
+                if (outer_terms) {
+                    Dfl db{0.f, 0.f};
+#pragma unroll
+                    for (int rb = 0; rb < 5; ++rb) {  // per window qubit
+                        float d = 0.f;
+                        if (rb >= r0 && rb < r1) {
+#pragma unroll
+                            for (int h = 0; h < 16; ++h) {
+                                const float2 v = halves(imconj(rb == 4 ? swap(x[h]) : x[h ^ ((1 << rb) & 15)], ph[h]));
+                                d += v.x;
+                                uv[h] = v.y;
+                            }
+#pragma unroll
+                            for (int h = 0; h < 16; ++h) d += uv[h];
+                        }
+                        dfl_add(db, d);
                     }
-                }
-                Dfl db{0.f, 0.f};
+                    for (int q = L.x0; q < L.x1; ++q) {  // outer qubits outside the window
+                        const MT w = base ^ MT(C->col[q]);
+                        float t = 0.f;
 #pragma unroll
-                for (int rb = 0; rb < 5; ++rb) dfl_add(db, dq[rb]);
-                for (int q = L.x0; q < (outer_terms ? L.x1 : L.x0); ++q) {  // outer qubits outside the window
-                    const uint64_t cq = C->col[q];
-                    float t = 0.f;
+                        for (int h = 0; h < 16; ++h) {
+                            int cl, cu;
+                            const float2 v = halves(imconj(x[h], phase(w, h, cl, cu)));
+                            t += v.x;
+                            uv[h] = v.y;
+                        }
 #pragma unroll
-                    for (int i = 0; i < 32; ++i)
-                        t += imconj(x[i], __ldg(lut + __popcll(lo[i & 3] ^ hi[i >> 2] ^ cq)));
-                    dfl_add(db, t);
+                        for (int h = 0; h < 16; ++h) t += uv[h];
+                        dfl_add(db, t);
+                    }
+                    dfl_add(s_db, db);
                 }
-                // lambda = 2^(-n/2) kappa_1^(2 n_in) x once the first mixer is undone
-                const float wgt2 = 2.f * float(C->weight) * mult * __int_as_float((127 - C->n) << 23) * f1.k2n;
-                add_gp(Dfl{dg, 0.f}, wgt2, L.grad, gj * 2 * p);
-                if (outer_terms) add_gp(db, wgt2, L.grad, gj * 2 * p + p);
+            } else {
+                P2 x[32];
+                if (MODE == kOuterGen) {
+                    const float2 *tab = reinterpret_cast<const float2 *>(s_tab[warp]);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) x[i] = load_amp(tab + popc_w(MT(lo[i & 3] ^ wh[i >> 2] ^ base)));
+                    first_mix_regs<32, false, LO>(x, r0, r1, f1);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) x[i] = load_amp(sp + (int64_t(i) << b));
+                    if (L.sign > 0)
+                        first_mix_regs<32, false, LO>(x, r0, r1, f1);
+                    else
+                        first_mix_regs<32, true, LO>(x, r0, r1, f1);
+                }
+#pragma unroll
+                for (int i = 0; i < 32; ++i) store_amp(sp + (int64_t(i) << b), x[i]);
             }
         }
-        if (MODE != kOuterFirst) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) sp[int64_t(i) << b] = x[i];
+        if (MODE == kOuterFirst) {
+            // lambda = 2^(-n/2) kappa_1^(2 n_in) x once the first mixer is undone
+            const float wgt2 = 2.f * float(C->weight) * mult * __int_as_float((127 - C->n) << 23) * f1.k2n;
+            add_gp(s_dg, wgt2, L.grad, gj * 2 * p);
+            if (p > 1) add_gp(s_db, wgt2, L.grad, gj * 2 * p + p);
         }
     }
 }
@@ -747,75 +813,77 @@ __device__ __forceinline__ int spread_slot(int slot, int pos, int gn) {
     return (slot & ((1 << pos) - 1)) | ((slot >> pos) << (pos + gn));
 }
 
-// First-layer cut words of a chunk slot: `base` for the slot's fixed bits,
-// lo/hi over the G register qubits w0 .. w0+G-1.
-template <int G>
-__device__ __forceinline__ void slot_words(const DevCone *__restrict__ C, uint64_t base, int w0, uint64_t (&lo)[4],
-                                           uint64_t (&hi)[8]) {
-    uint64_t cr[5];
+// What the slots of a chunk share, in shared memory: the first layer's phase
+// table and the cut words of the chunk's 13 bits.
+template <typename MT>
+struct ChunkItem {
+    float2 tab[kOuterRow];
+    MT col[kChunkBits];
+};
+
+// First-layer cut words over the G register bits from chunk bit pos on: lo over
+// the first two, hi over the rest, with the slot's fixed bits sb and cw.
+template <int G, typename MT>
+__device__ __forceinline__ void slot_words(const ChunkItem<MT> &I, MT cw, int sb, int pos, MT (&lo)[4], MT (&hi)[8]) {
+    MT base = cw;
 #pragma unroll
-    for (int b = 0; b < 5; ++b) cr[b] = b < G ? C->col[w0 + b] : 0ull;
+    for (int b = 0; b < kChunkBits; ++b)
+        if ((sb >> b) & 1) base ^= I.col[b];  // the register bits of sb are zero
+    MT cr[5];
+#pragma unroll
+    for (int b = 0; b < 5; ++b) cr[b] = b < G ? I.col[pos + b] : MT(0);
     lo[0] = 0;
     lo[1] = cr[0];
     lo[2] = cr[1];
     lo[3] = cr[0] ^ cr[1];
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-        hi[k] = base ^ ((k & 1) ? cr[2] : 0ull) ^ ((k & 2) ? cr[3] : 0ull) ^ ((k & 4) ? cr[4] : 0ull);
+        hi[k] = base ^ ((k & 1) ? cr[2] : MT(0)) ^ ((k & 2) ? cr[3] : MT(0)) ^ ((k & 4) ? cr[4] : MT(0));
 }
 
 // One round of a chunk pass: every slot gathers the 2^G amplitudes that
 // differ in chunk bits [pos, pos+G), applies the mixer to those G qubits and
 // writes them back.  GEN in its first round generates the amplitudes instead.
-template <int G, bool GEN>
-__device__ __forceinline__ void chunk_round(float2 *__restrict__ sm, int n_el, int pos, FirstMix f, bool inv,
-                                            const DevCone *__restrict__ C, uint64_t cw, int lo_bits, int RB, int w0,
-                                            const float2 *__restrict__ lut, bool rd_swz, bool wr_swz) {
+template <int G, bool GEN, bool INV, bool LO, typename MT>
+__device__ __forceinline__ void chunk_round(float2 *__restrict__ sm, int n_el, int pos, const FirstMix &f,
+                                            const ChunkItem<MT> &I, MT cw, bool rd_swz, bool wr_swz) {
     constexpr int NR = 1 << G;
     for (int slot = threadIdx.x; slot < (n_el >> G); slot += kChunkThreads) {
         const int sb = spread_slot(slot, pos, G);
-        float2 x[NR];
+        P2 x[NR];
         if (GEN) {
-            uint64_t base = cw;
-            for (int b = 0; b < lo_bits; ++b)  // the window bits of sb are zero in the first round
-                if ((sb >> b) & 1) base ^= C->col[qubit_of(b, RB)];
-            for (int b = lo_bits + G; b < kChunkBits; ++b)
-                if ((sb >> b) & 1) base ^= C->col[w0 + b - lo_bits];
-            uint64_t lo[4], hi[8];
-            slot_words<G>(C, base, w0, lo, hi);
+            MT lo[4], hi[8];
+            slot_words<G>(I, cw, sb, pos, lo, hi);
 #pragma unroll
-            for (int i = 0; i < NR; ++i) x[i] = __ldg(lut + __popcll(lo[i & 3] ^ hi[i >> 2]));
+            for (int i = 0; i < NR; ++i) x[i] = load_amp(I.tab + popc_w(MT(lo[i & 3] ^ hi[i >> 2])));
         } else {
 #pragma unroll
-            for (int i = 0; i < NR; ++i) x[i] = sm[sidx(sb | (i << pos), rd_swz)];
+            for (int i = 0; i < NR; ++i) x[i] = load_amp(sm + sidx(sb | (i << pos), rd_swz));
         }
-        if (inv)
-            first_mix_regs<NR, true>(x, 0, G, f);
-        else
-            first_mix_regs<NR, false>(x, 0, G, f);
+        first_mix_regs<NR, INV, LO>(x, 0, G, f);
 #pragma unroll
-        for (int i = 0; i < NR; ++i) sm[sidx(sb | (i << pos), wr_swz)] = x[i];
+        for (int i = 0; i < NR; ++i) store_amp(sm + sidx(sb | (i << pos), wr_swz), x[i]);
     }
 }
 
-template <bool GEN>
-__device__ __forceinline__ void chunk_round_any(int G, float2 *sm, int n_el, int pos, FirstMix f, bool inv,
-                                                const DevCone *C, uint64_t cw, int lo_bits, int RB, int w0,
-                                                const float2 *lut, bool rd_swz, bool wr_swz) {
+template <bool GEN, bool INV, bool LO, typename MT>
+__device__ __forceinline__ void chunk_round_any(int G, float2 *sm, int n_el, int pos, const FirstMix &f,
+                                                const ChunkItem<MT> &I, MT cw, bool rd_swz, bool wr_swz) {
     switch (G) {
-        case 1: chunk_round<1, GEN>(sm, n_el, pos, f, inv, C, cw, lo_bits, RB, w0, lut, rd_swz, wr_swz); break;
-        case 2: chunk_round<2, GEN>(sm, n_el, pos, f, inv, C, cw, lo_bits, RB, w0, lut, rd_swz, wr_swz); break;
-        case 3: chunk_round<3, GEN>(sm, n_el, pos, f, inv, C, cw, lo_bits, RB, w0, lut, rd_swz, wr_swz); break;
-        case 4: chunk_round<4, GEN>(sm, n_el, pos, f, inv, C, cw, lo_bits, RB, w0, lut, rd_swz, wr_swz); break;
-        default: chunk_round<5, GEN>(sm, n_el, pos, f, inv, C, cw, lo_bits, RB, w0, lut, rd_swz, wr_swz); break;
+        case 1: chunk_round<1, GEN, INV, LO>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
+        case 2: chunk_round<2, GEN, INV, LO>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
+        case 3: chunk_round<3, GEN, INV, LO>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
+        case 4: chunk_round<4, GEN, INV, LO>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
+        default: chunk_round<5, GEN, INV, LO>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
     }
 }
 
-template <int MODE>
+template <int MODE, bool LO, typename MT>
 __global__ void __launch_bounds__(kChunkThreads, 2)
     split_chunk_kernel(const __grid_constant__ BigLaunch L, const __grid_constant__ CUtensorMap tmap) {
     extern __shared__ __align__(1024) float2 sm[];
     __shared__ uint64_t s_bar;  // completion of the chunk's load
+    __shared__ ChunkItem<MT> s_item;
     const int tid = threadIdx.x;
     if (tid == 0) mbar_init(&s_bar);
     __syncthreads();
@@ -840,7 +908,6 @@ __global__ void __launch_bounds__(kChunkThreads, 2)
         }
         const int64_t gj = int64_t(C->graph) * L.P + j;
         const FirstMix f1 = first_mix(L, gj, nin);
-        const bool inv = MODE == kOuterFirst || (MODE == kOuterMix && L.sign < 0);
         // element e of the chunk <-> address xb + (e & runmask) + ((e >> lo_bits) << w0) of
         // item it; tensor coordinates: run, middle bits, window (two dimensions), high bits x item
         const int64_t xb = ((ch & lowmask) << lo_bits) | ((ch >> (w0 - lo_bits)) << (w0 + w));
@@ -850,14 +917,18 @@ __global__ void __launch_bounds__(kChunkThreads, 2)
             fence_async_smem();  // the previous task's accesses come before the copy's writes
             tma_load(&tmap, sm, &s_bar, uint32_t(n_el * sizeof(float2)), crd);
         }
-        // cut word of the chunk's fixed bits (shell block and address bits outside the chunk)
+        // the item's table and the chunk bits' cut words, and the cut word of its
+        // fixed bits (shell block and address bits outside the chunk)
         float mult = 1.f;
-        uint64_t cw = 0;
-        const float2 *__restrict__ lut = L.lut + gj * p * L.cmax1;  // first layer's phase table
+        MT cw = 0;
         if (MODE != kOuterMix) {
-            cw = shell_block(C, L.shell, uint32_t(y), mult);
+            const float2 *__restrict__ lut = L.lut + gj * p * L.cmax1;  // first layer's phase table
+            for (int e = tid; e < L.cmax1; e += kChunkThreads) s_item.tab[e] = __ldg(lut + e);
+            if (tid < kChunkBits)
+                s_item.col[tid] = MT(C->col[tid < lo_bits ? qubit_of(tid, RB) : w0 + tid - lo_bits]);
+            cw = MT(shell_block(C, L.shell, uint32_t(y), mult));
             for (int a = lo_bits; a < nin; ++a)
-                if ((a < w0 || a >= w0 + w) && ((xb >> a) & 1)) cw ^= C->col[qubit_of(a, RB)];
+                if ((a < w0 || a >= w0 + w) && ((xb >> a) & 1)) cw ^= MT(C->col[qubit_of(a, RB)]);
         }
         if (MODE != kOuterGen) {
             // bounded wait; should it ever run out (never expected), record it,
@@ -877,17 +948,18 @@ __global__ void __launch_bounds__(kChunkThreads, 2)
             const bool swz_on = lo_bits < 4;
             const bool rd_swz = swz_on && g0 > 0, wr_swz = swz_on && (g0 + gn < w || MODE == kOuterFirst);
             if (MODE == kOuterGen && g0 == 0)
-                chunk_round_any<true>(gn, sm, n_el, lo_bits, f1, false, C, cw, lo_bits, RB, w0, lut, rd_swz, wr_swz);
+                chunk_round_any<true, false, LO>(gn, sm, n_el, lo_bits, f1, s_item, cw, rd_swz, wr_swz);
+            else if (MODE == kOuterGen || (MODE == kOuterMix && L.sign > 0))
+                chunk_round_any<false, false, LO>(gn, sm, n_el, lo_bits + g0, f1, s_item, cw, rd_swz, wr_swz);
             else
-                chunk_round_any<false>(gn, sm, n_el, lo_bits + g0, f1, inv, C, cw, lo_bits, RB, w0, lut, rd_swz,
-                                       wr_swz);
+                chunk_round_any<false, true, LO>(gn, sm, n_el, lo_bits + g0, f1, s_item, cw, rd_swz, wr_swz);
             __syncthreads();
         }
         if (MODE == kOuterFirst) {
             // lambda is now fully un-mixed: the first layer's phase term and the
             // outer qubits' mixer terms against exp(-i gamma_1 C)|+>
             const bool outer_terms = p > 1;
-            const float c0 = 0.5f * float(C->m);  // Im<lambda|psi> = 0: C - c0 in place of C
+            const float b0 = 4194304.f + 0.5f * float(C->m);  // Im<lambda|psi> = 0: C - c0 in place of C
             const int gn = min(5, w);
             const int nreg = 1 << gn;
             Dfl dg{0.f, 0.f}, db{0.f, 0.f};  // this thread's slots, compensated
@@ -897,19 +969,14 @@ __global__ void __launch_bounds__(kChunkThreads, 2)
 #pragma unroll
                 for (int i = 0; i < 32; ++i)
                     x[i] = i < nreg ? sm[sidx(sb | (i << lo_bits), lo_bits < 4)] : make_float2(0.f, 0.f);
-                uint64_t base = cw;
-                for (int b = 0; b < lo_bits; ++b)
-                    if ((sb >> b) & 1) base ^= C->col[qubit_of(b, RB)];
-                for (int b = lo_bits + gn; b < kChunkBits; ++b)
-                    if ((sb >> b) & 1) base ^= C->col[w0 + b - lo_bits];
-                uint64_t lo[4], hi[8];
-                slot_words<5>(C, base, w0, lo, hi);  // w > 5 here: five window qubits in registers
+                MT lo[4], hi[8];
+                slot_words<5>(s_item, cw, sb, lo_bits, lo, hi);  // w > 5 here: five window qubits in registers
                 float dgs = 0.f, dq[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
-                    const int c = __popcll(lo[i & 3] ^ hi[i >> 2]);
-                    const float2 ph = __ldg(lut + c);
-                    dgs = fmaf(float(c) - c0, imconj(x[i], ph), dgs);
+                    const int c = popc_w(MT(lo[i & 3] ^ hi[i >> 2]));
+                    const float2 ph = s_item.tab[c];
+                    dgs = fmaf(cut_minus(c, b0), imconj(x[i], ph), dgs);
                     if (outer_terms) {
 #pragma unroll
                         for (int rb = 0; rb < 5; ++rb) dq[rb] += imconj(x[i ^ (1 << rb)], ph);
@@ -921,11 +988,11 @@ __global__ void __launch_bounds__(kChunkThreads, 2)
                     for (int rb = 0; rb < 5; ++rb) dfl_add(db, dq[rb]);
                     // the other outer qubits: the rest of the window, then beyond it
                     for (int q = w0 + 5; q < L.x1; ++q) {
-                        const uint64_t cq = C->col[q];
+                        const MT cq = MT(C->col[q]);
                         float t = 0.f;
 #pragma unroll
                         for (int i = 0; i < 32; ++i)
-                            t += imconj(x[i], __ldg(lut + __popcll(lo[i & 3] ^ hi[i >> 2] ^ cq)));
+                            t += imconj(x[i], s_item.tab[popc_w(MT(lo[i & 3] ^ hi[i >> 2] ^ cq))]);
                         dfl_add(db, t);
                     }
                 }
@@ -996,25 +1063,48 @@ bool split_ok(int n_in, int p, const int32_t *k, bool grad) {
     return true;
 }
 
+namespace {
+
+// The variants of a pass: lo, the first mixer's coefficient as a hi + lo pair (the
+// adjoint's passes); wide, 64-bit cut words.  kOuterFirst is the adjoint's alone.
+template <int MODE, bool LO>
+const void *outer_fn(bool wide) {
+    return wide ? (const void *)split_outer_kernel<MODE, LO, uint64_t> : (const void *)split_outer_kernel<MODE, LO, uint32_t>;
+}
+const void *outer_fn(int mode, bool lo, bool wide) {
+    if (mode == kOuterGen) return lo ? outer_fn<kOuterGen, true>(wide) : outer_fn<kOuterGen, false>(wide);
+    if (mode == kOuterMix) return lo ? outer_fn<kOuterMix, true>(false) : outer_fn<kOuterMix, false>(false);
+    return outer_fn<kOuterFirst, true>(wide);
+}
+template <int MODE, bool LO>
+const void *chunk_fn(bool wide) {
+    return wide ? (const void *)split_chunk_kernel<MODE, LO, uint64_t> : (const void *)split_chunk_kernel<MODE, LO, uint32_t>;
+}
+const void *chunk_fn(int mode, bool lo, bool wide) {
+    if (mode == kOuterGen) return lo ? chunk_fn<kOuterGen, true>(wide) : chunk_fn<kOuterGen, false>(wide);
+    if (mode == kOuterMix) return lo ? chunk_fn<kOuterMix, true>(false) : chunk_fn<kOuterMix, false>(false);
+    return chunk_fn<kOuterFirst, true>(wide);
+}
+
+constexpr size_t kChunkSmem = sizeof(float2) << kChunkBits;
+
+}  // namespace
+
 // Chunk kernels need more than the default 48 KB of dynamic shared memory:
-// raised once per kernel and device.
-static cudaError_t allow_chunk_smem(const void *fn, int mode) {
+// raised once per device, at upload.
+cudaError_t split_prepare() {
     static std::mutex mu;
-    static std::set<std::pair<int, int>> done;
+    static std::set<int> done;
     int dev = 0;
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk(mu);
-    if (done.count({dev, mode})) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(sizeof(float2) << kChunkBits));
-    if (e == cudaSuccess) done.insert({dev, mode});
-    return e;
-}
-
-cudaError_t split_prepare() {
-    cudaError_t e = allow_chunk_smem((const void *)split_chunk_kernel<kOuterGen>, kOuterGen);
-    if (e == cudaSuccess) e = allow_chunk_smem((const void *)split_chunk_kernel<kOuterMix>, kOuterMix);
-    if (e == cudaSuccess) e = allow_chunk_smem((const void *)split_chunk_kernel<kOuterFirst>, kOuterFirst);
+    if (done.count(dev)) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    for (int mode : {kOuterGen, kOuterMix, kOuterFirst})
+        for (int v = 0; v < 4 && e == cudaSuccess; ++v)
+            e = cudaFuncSetAttribute(chunk_fn(mode, v & 1, v & 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     int(kChunkSmem));
+    if (e == cudaSuccess) done.insert(dev);
     return e;
 }
 
@@ -1036,9 +1126,14 @@ cudaError_t launch_split_wave(BigLaunch B, bool grad, int chunk_window, int64_t 
         win.push_back({w0, w0 + n, left > 5});
         w0 += n;
     }
-    auto grid_for = [](const void *fn, int64_t tasks) {
-        const int64_t need = std::max<int64_t>(1, (tasks + 3) / 4);
-        return int(std::min<int64_t>(occupancy_grid(fn, 128, 0), need));
+    // tiles per warp task (2^tile_bits tiles per item): as many as leave two tasks
+    // for every resident warp of 4 * blocks (of 1, 2, 4, 8, 16 tasks: 9.46, 8.77,
+    // 8.94, 9.02, 9.37 ms on the 6x6 torus at p = 3, energy, 32 points; within 3%
+    // for four cubic graphs n = 24, gradient)
+    auto tiles_per_task = [](int64_t items, int tile_bits, int blocks) {
+        int t = 1;
+        while (t < (1 << std::min(tile_bits, 6)) && (items << tile_bits) / (2 * t) >= int64_t(blocks) * 4 * 2) t *= 2;
+        return t;
     };
     auto outer = [&](int mode, size_t w, int sign) -> cudaError_t {
         B.mode = mode;
@@ -1048,34 +1143,25 @@ cudaError_t launch_split_wave(BigLaunch B, bool grad, int chunk_window, int64_t 
         B.x0 = win[w].w1;
         B.x1 = nin;
         B.sign = sign;
+        const bool wide = B.cmax1 - 1 > 32;
         if (win[w].chunk) {
-            const size_t smem = size_t(sizeof(float2)) << kChunkBits;
             CUtensorMap map;
             if (cudaError_t e = chunk_map(B, B.w0, B.w1 - B.w0, &map); e != cudaSuccess) return e;
             const int64_t tasks = B.n_items << (nin - kChunkBits);
-            const void *fn = mode == kOuterGen   ? (const void *)split_chunk_kernel<kOuterGen>
-                             : mode == kOuterMix ? (const void *)split_chunk_kernel<kOuterMix>
-                                                 : (const void *)split_chunk_kernel<kOuterFirst>;
-            if (cudaError_t e = allow_chunk_smem(fn, mode); e != cudaSuccess) return e;
-            const int grid = int(std::min<int64_t>(occupancy_grid(fn, kChunkThreads, smem), std::max<int64_t>(tasks, 1)));
-            if (mode == kOuterGen)
-                split_chunk_kernel<kOuterGen><<<grid, kChunkThreads, smem, s>>>(B, map);
-            else if (mode == kOuterMix)
-                split_chunk_kernel<kOuterMix><<<grid, kChunkThreads, smem, s>>>(B, map);
-            else
-                split_chunk_kernel<kOuterFirst><<<grid, kChunkThreads, smem, s>>>(B, map);
+            const void *fn = chunk_fn(mode, grad, wide);
+            const int grid = int(std::min<int64_t>(occupancy_grid(fn, kChunkThreads, kChunkSmem), std::max<int64_t>(tasks, 1)));
+            void *args[] = {&B, &map};
+            if (cudaError_t e = cudaLaunchKernel(fn, dim3(unsigned(grid)), dim3(kChunkThreads), args, kChunkSmem, s);
+                e != cudaSuccess)
+                return e;
         } else {
-            const int64_t tasks = B.n_items << (nin - 10);
-            if (mode == kOuterGen) {
-                const void *fn = (const void *)split_outer_kernel<kOuterGen>;
-                split_outer_kernel<kOuterGen><<<grid_for(fn, tasks), 128, 0, s>>>(B);
-            } else if (mode == kOuterMix) {
-                const void *fn = (const void *)split_outer_kernel<kOuterMix>;
-                split_outer_kernel<kOuterMix><<<grid_for(fn, tasks), 128, 0, s>>>(B);
-            } else {
-                const void *fn = (const void *)split_outer_kernel<kOuterFirst>;
-                split_outer_kernel<kOuterFirst><<<grid_for(fn, tasks), 128, 0, s>>>(B);
-            }
+            const void *fn = outer_fn(mode, grad, wide);
+            const int full = occupancy_grid(fn, 128, 0);
+            B.tpw = tiles_per_task(B.n_items, nin - 10, full);
+            const int64_t tasks = (B.n_items << (nin - 10)) / B.tpw;
+            const int grid = int(std::min<int64_t>(full, std::max<int64_t>(1, (tasks + 3) / 4)));
+            void *args[] = {&B};
+            if (cudaError_t e = cudaLaunchKernel(fn, dim3(unsigned(grid)), dim3(128), args, 0, s); e != cudaSuccess) return e;
         }
         ++launches;
         return cudaGetLastError();
@@ -1085,15 +1171,11 @@ cudaError_t launch_split_wave(BigLaunch B, bool grad, int chunk_window, int64_t 
     for (size_t w = 0; w < win.size() && e == cudaSuccess; ++w) e = outer(w == 0 ? kOuterGen : kOuterMix, w, 1);
     if (e != cudaSuccess) return e;
     B.load = win.empty() ? 0 : 1;
-    // tiles per warp task: as many as leave two tasks for every resident warp (of 1, 2, 4, 8, 16: 9.46, 8.77, 8.94,
-    // 9.02, 9.37 ms on the 6x6 torus at p = 3, energy, 32 points; within 3% for four cubic graphs n = 24, gradient)
     const void *core = grad ? (const void *)split_core_kernel<true, kSplitRbGrad>
                             : (const void *)split_core_kernel<false, kSplitRbEnergy>;
     const size_t core_smem = core_smem_bytes(p, grad);
     const int core_grid = occupancy_grid(core, 128, core_smem);
-    B.tpw = 1;
-    while (B.tpw < (1 << std::min(nin - T, 6)) && (B.n_items << (nin - T)) / (2 * B.tpw) >= int64_t(core_grid) * 4 * 2)
-        B.tpw *= 2;
+    B.tpw = tiles_per_task(B.n_items, nin - T, core_grid);
     const int64_t core_tasks = (B.n_items << (nin - T)) / B.tpw;
     const int grid = int(std::min<int64_t>(core_grid, std::max<int64_t>(1, (core_tasks + 3) / 4)));
     if (grad)
