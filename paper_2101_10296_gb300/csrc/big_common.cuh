@@ -3,20 +3,145 @@
 
 #include "big.cuh"
 #include "dev_math.cuh"
+#include "packed.cuh"
 
 namespace qaoa {
 namespace {
 
-// c me - i s other: one output of exp(-i beta X) on the pair (me, other),
-// with c = cs.x + cs.z and s = cs.y + cs.w (hi and lo FP32 parts)
-__device__ __forceinline__ float2 rot(float2 me, float2 o, float4 cs) {
-    return make_float2(fmaf(cs.x, me.x, fmaf(cs.y, o.y, fmaf(cs.z, me.x, cs.w * o.y))),
-                       fmaf(cs.x, me.y, fmaf(-cs.y, o.x, fmaf(cs.z, me.y, -cs.w * o.x))));
+// One output of exp(-i beta X) on the pair (me, o), c me - i s o, or of
+// exp(+i beta X) (INV), with c = cs.x + cs.z and s = cs.y + cs.w (hi and lo FP32
+// parts), on the amplitudes of two packed registers.
+template <bool INV>
+__device__ __forceinline__ C2 rot2(const C2 &me, const C2 &o, float4 cs) {
+    const float s = INV ? -cs.y : cs.y, w = INV ? -cs.w : cs.w;
+    return C2{fma2(splat(cs.x), me.r, fma2(splat(s), o.i, fma2(splat(cs.z), me.r, mul2(splat(w), o.i)))),
+              fma2(splat(cs.x), me.i, fma2(splat(-s), o.r, fma2(splat(cs.z), me.i, mul2(splat(-w), o.r))))};
 }
-// the same for exp(+i beta X)
-__device__ __forceinline__ float2 unrot(float2 me, float2 o, float4 cs) {
-    return make_float2(fmaf(cs.x, me.x, fmaf(-cs.y, o.y, fmaf(cs.z, me.x, -cs.w * o.y))),
-                       fmaf(cs.x, me.y, fmaf(cs.y, o.x, fmaf(cs.z, me.y, cs.w * o.x))));
+
+// The same (forward) on one amplitude, its real and imaginary parts a packed pair.
+__device__ __forceinline__ P2 rot1(P2 me, P2 o, float4 cs) {
+    const P2 so = swap(o);
+    return fma2(splat(cs.x), me, fma2(p2(cs.y, -cs.y), so, fma2(splat(cs.z), me, mul2(p2(cs.w, -cs.w), so))));
+}
+
+// op(me, partner) on register qubit q of a tile
+template <int NP, class F>
+__device__ __forceinline__ void on_reg(C2 (&x)[NP], int q, F &&op) {
+    if ((1 << q) == NP) {
+#pragma unroll
+        for (int h = 0; h < NP; ++h) x[h] = op(x[h], swap(x[h]));
+    } else {
+#pragma unroll
+        for (int h = 0; h < NP; ++h) {
+            if (h & (1 << q)) continue;
+            const int j = h | (1 << q);
+            const C2 u = x[h], v = x[j];
+            x[h] = op(u, v);
+            x[j] = op(v, u);
+        }
+    }
+}
+
+// Im<r|X_q|x> over register qubit q: the pairs' terms in register order.
+template <int NP>
+__device__ __forceinline__ float xterm_reg(const C2 (&x)[NP], const C2 (&r)[NP], int q) {
+    float d = 0.f;
+    if ((1 << q) == NP) {
+#pragma unroll
+        for (int h = 0; h < NP; ++h) {
+            const float2 t = halves(imconj(r[h], swap(x[h])));
+            d += t.x + t.y;
+        }
+    } else {
+        float up[NP / 2];
+        int n = 0;
+#pragma unroll
+        for (int h = 0; h < NP; ++h) {
+            if (h & (1 << q)) continue;
+            const int j = h | (1 << q);
+            const float2 t = halves(add2(imconj(r[h], x[j]), imconj(r[j], x[h])));
+            d += t.x;
+            up[n++] = t.y;
+        }
+#pragma unroll
+        for (int k = 0; k < NP / 2; ++k) d += up[k];
+    }
+    return d;
+}
+
+// The same over a lane qubit, given the partner's x.
+template <int NP>
+__device__ __forceinline__ float xterm_lane(const C2 (&xo)[NP], const C2 (&r)[NP]) {
+    float d = 0.f, up[NP];
+#pragma unroll
+    for (int h = 0; h < NP; ++h) {
+        const float2 t = halves(imconj(r[h], xo[h]));
+        d += t.x;
+        up[h] = t.y;
+    }
+#pragma unroll
+    for (int h = 0; h < NP; ++h) d += up[h];
+    return d;
+}
+
+// An amplitude as a packed pair.
+__device__ __forceinline__ P2 load_amp(const float2 *p) { return P2{*reinterpret_cast<const unsigned long long *>(p)}; }
+__device__ __forceinline__ void store_amp(float2 *p, P2 v) { *reinterpret_cast<unsigned long long *>(p) = v.v; }
+
+// Cut words as 32 bits where every cone of the plan fits them, else 64.
+__device__ __forceinline__ int popc_w(uint32_t x) { return __popc(x); }
+__device__ __forceinline__ int popc_w(uint64_t x) { return __popcll(x); }
+// XOR over the lanes.
+__device__ __forceinline__ uint32_t warp_xor(uint32_t x) { return __reduce_xor_sync(kFull, x); }
+__device__ __forceinline__ uint64_t warp_xor(uint64_t x) {
+    return (uint64_t(__reduce_xor_sync(kFull, uint32_t(x >> 32))) << 32) | __reduce_xor_sync(kFull, uint32_t(x));
+}
+// c - c0 of a cut value, given b0 = 2^22 + c0 (halves are exact at that size)
+__device__ __forceinline__ float cut_minus(int c, float b0) { return __uint_as_float(0x4A800000u + 2u * uint32_t(c)) - b0; }
+
+__device__ __forceinline__ float lds1(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void opaque(uint32_t &v) { asm volatile("" : "+r"(v)); }
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return uint32_t(__cvta_generic_to_shared(p)); }
+
+// Rows of a warp's phase tables: 68 real parts, then 68 imaginary parts (a cone
+// has at most 64 cut bits); count bytes hold 2 c.
+constexpr int kCoreRow = 544, kCoreIm = 272;
+constexpr float kCoreScale = 2.f;
+// Stages p layers' phase tables in rows (above); called by the whole warp.
+__device__ __forceinline__ void stage_rows(unsigned char *tab, const float2 *__restrict__ lut, int p, int cmax1, int lane) {
+    for (int l = 0; l < p; ++l)
+        for (int e = lane; e < cmax1; e += 32) {
+            const float2 v = __ldg(lut + l * cmax1 + e);
+            *reinterpret_cast<float *>(tab + l * kCoreRow + 4 * e) = v.x;
+            *reinterpret_cast<float *>(tab + l * kCoreRow + kCoreIm + 4 * e) = v.y;
+        }
+}
+// Entries of count byte a of two packed words in a row.
+__device__ __forceinline__ C2 row_entry(uint32_t row, uint32_t wa, uint32_t wb, int a) {
+    const uint32_t p = row + (__byte_perm(wa, 0u, 0x4440u | uint32_t(a)) << 1);
+    const uint32_t q = row + (__byte_perm(wb, 0u, 0x4440u | uint32_t(a)) << 1);
+    return C2{p2(lds1(p), lds1(q)), p2(lds1(p + kCoreIm), lds1(q + kCoreIm))};
+}
+// kCoreScale (c - c0) of the same bytes, given b0 = 2^23 + kCoreScale c0.
+__device__ __forceinline__ P2 row_weight(uint32_t wa, uint32_t wb, int a, float b0) {
+    return add2(p2(__uint_as_float(__byte_perm(wa, 0x4B000000u, 0x7540u | uint32_t(a))),
+                   __uint_as_float(__byte_perm(wb, 0x4B000000u, 0x7540u | uint32_t(a)))),
+                splat(-b0));
+}
+// Amplitudes at offsets i and j of p in one packed register.
+__device__ __forceinline__ C2 load_pair(const float2 *p, int64_t i, int64_t j) {
+    const float2 u = p[i], v = p[j];
+    return C2{p2(u.x, v.x), p2(u.y, v.y)};
+}
+__device__ __forceinline__ void store_pair(float2 *p, int64_t i, int64_t j, const C2 &x) {
+    const float2 a = halves(x.r), b = halves(x.i);
+    p[i] = make_float2(a.x, b.x);
+    p[j] = make_float2(a.y, b.y);
 }
 
 // Warp sum in FP32 (every lane gets it).

@@ -38,7 +38,6 @@
 
 #include "big.cuh"
 #include "big_common.cuh"
-#include "packed.cuh"
 
 namespace qaoa {
 namespace {
@@ -129,37 +128,12 @@ __device__ __forceinline__ void first_mix_regs(P2 (&x)[NR], int r0, int r1, cons
         fmix_regs<NR, false, INV, LO>(x, r0, r1, f.a, f.alo);
 }
 
-// An amplitude as a packed pair.
-__device__ __forceinline__ P2 load_amp(const float2 *p) { return P2{*reinterpret_cast<const unsigned long long *>(p)}; }
-__device__ __forceinline__ void store_amp(float2 *p, P2 v) { *reinterpret_cast<unsigned long long *>(p) = v.v; }
-
-// Cut words as 32 bits where every cone of the plan fits them, else 64.
-__device__ __forceinline__ int popc_w(uint32_t x) { return __popc(x); }
-__device__ __forceinline__ int popc_w(uint64_t x) { return __popcll(x); }
-// XOR over the lanes.
-__device__ __forceinline__ uint32_t warp_xor(uint32_t x) { return __reduce_xor_sync(kFull, x); }
-__device__ __forceinline__ uint64_t warp_xor(uint64_t x) {
-    return (uint64_t(__reduce_xor_sync(kFull, uint32_t(x >> 32))) << 32) | __reduce_xor_sync(kFull, uint32_t(x));
-}
-// c - c0 of a cut value, given b0 = 2^22 + c0 (halves are exact at that size)
-__device__ __forceinline__ float cut_minus(int c, float b0) { return __uint_as_float(0x4A800000u + 2u * uint32_t(c)) - b0; }
-
-__device__ __forceinline__ uint32_t smem_addr(const void *p) { return uint32_t(__cvta_generic_to_shared(p)); }
-
 // ---------------------------------------------------------------- core pass
 // The tile in packed FP32x2 pairs (packed.cuh): C2 number h holds registers h
 // and h + NR/2, every operation of the sweep is one instruction for both, and
 // the highest register qubit's partner is the other half.  Sums that run over
 // the registers in order (the observable, the derivative terms) take the lower
 // halves first, then the upper ones.
-
-// c me - i s o (rot) or c me + i s o (unrot), see big_common.cuh
-template <bool INV>
-__device__ __forceinline__ C2 rot2(const C2 &me, const C2 &o, float4 cs) {
-    const float s = INV ? -cs.y : cs.y, w = INV ? -cs.w : cs.w;
-    return C2{fma2(splat(cs.x), me.r, fma2(splat(s), o.i, fma2(splat(cs.z), me.r, mul2(splat(w), o.i)))),
-              fma2(splat(cs.x), me.i, fma2(splat(-s), o.r, fma2(splat(cs.z), me.i, mul2(splat(-w), o.r))))};
-}
 
 // fmix on two amplitudes
 template <bool B, bool INV, bool LO>
@@ -171,24 +145,6 @@ __device__ __forceinline__ C2 fmix2(const C2 &me, const C2 &o, float a, float al
     }
     const P2 px = LO ? fma2(splat(alo), me.r, oi) : oi, py = LO ? fma2(splat(alo), me.i, nor) : nor;
     return C2{fma2(splat(a), me.r, px), fma2(splat(a), me.i, py)};
-}
-
-// op(me, partner) on register qubit q of a tile
-template <int NP, class F>
-__device__ __forceinline__ void on_reg(C2 (&x)[NP], int q, F &&op) {
-    if ((1 << q) == NP) {
-#pragma unroll
-        for (int h = 0; h < NP; ++h) x[h] = op(x[h], swap(x[h]));
-    } else {
-#pragma unroll
-        for (int h = 0; h < NP; ++h) {
-            if (h & (1 << q)) continue;
-            const int j = h | (1 << q);
-            const C2 u = x[h], v = x[j];
-            x[h] = op(u, v);
-            x[j] = op(v, u);
-        }
-    }
 }
 
 // op on register qubits [0, nr) and lane qubits [0, nl)
@@ -212,57 +168,8 @@ __device__ __forceinline__ void first_mix2(C2 (&x)[NP], int nr, int nl, const Fi
         on_qubits<NP>(x, nr, nl, [&](const C2 &u, const C2 &v) { return fmix2<false, INV, LO>(u, v, f.a, f.alo); });
 }
 
-// Im<r|X_q|x> over register qubit q: the pairs' terms in register order.
-template <int NP>
-__device__ __forceinline__ float xterm_reg(const C2 (&x)[NP], const C2 (&r)[NP], int q) {
-    float d = 0.f;
-    if ((1 << q) == NP) {
-#pragma unroll
-        for (int h = 0; h < NP; ++h) {
-            const float2 t = halves(imconj(r[h], swap(x[h])));
-            d += t.x + t.y;
-        }
-    } else {
-        float up[NP / 2];
-        int n = 0;
-#pragma unroll
-        for (int h = 0; h < NP; ++h) {
-            if (h & (1 << q)) continue;
-            const int j = h | (1 << q);
-            const float2 t = halves(add2(imconj(r[h], x[j]), imconj(r[j], x[h])));
-            d += t.x;
-            up[n++] = t.y;
-        }
-#pragma unroll
-        for (int k = 0; k < NP / 2; ++k) d += up[k];
-    }
-    return d;
-}
-
-// The same over a lane qubit, given the partner's x.
-template <int NP>
-__device__ __forceinline__ float xterm_lane(const C2 (&xo)[NP], const C2 (&r)[NP]) {
-    float d = 0.f, up[NP];
-#pragma unroll
-    for (int h = 0; h < NP; ++h) {
-        const float2 t = halves(imconj(r[h], xo[h]));
-        d += t.x;
-        up[h] = t.y;
-    }
-#pragma unroll
-    for (int h = 0; h < NP; ++h) d += up[h];
-    return d;
-}
-
 // <Z_0 Z_1> sign of register i (qubits 0 and 1 are register bits 0 and 1).
 __host__ __device__ constexpr float zz_sign(int i) { return ((i ^ (i >> 1)) & 1) ? -1.f : 1.f; }
-
-__device__ __forceinline__ float lds1(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(v) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ void opaque(uint32_t &v) { asm volatile("" : "+r"(v)); }
 
 // Resident CTAs per SM.  Adjoint: 3 (168 registers, no spills; 2, 4 and 5:
 // 16.4, 17.4 and 18.8 against 15.8 ms on four cubic graphs n = 24, p = 3, 25
@@ -270,10 +177,6 @@ __device__ __forceinline__ void opaque(uint32_t &v) { asm volatile("" : "+r"(v))
 // ms on the 6x6 torus).
 constexpr int kCoreGradBlocks = 3, kCoreEnergyBlocks = 4;
 
-// Rows of a warp's phase tables: 68 real parts, then 68 imaginary parts (a cone
-// has at most 64 cut bits); count bytes hold 2 c.
-constexpr int kCoreRow = 544, kCoreIm = 272;
-constexpr float kCoreScale = 2.f;
 inline size_t core_smem_bytes(int p, bool grad) { return size_t(4) * (p * kCoreRow + (grad ? 2 * p * 32 * sizeof(float2) : 0)); }
 
 // A warp takes L.tpw consecutive tiles of one item: the item's decoding, its
@@ -321,13 +224,7 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
         const float4 *__restrict__ cs = L.cs + gj * p;
         __syncwarp();
         {
-            const float2 *__restrict__ lut = L.lut + gj * p * L.cmax1;
-            for (int l = 0; l < p; ++l)
-                for (int e = lane; e < L.cmax1; e += 32) {
-                    const float2 v = __ldg(lut + l * L.cmax1 + e);
-                    *reinterpret_cast<float *>(tab + l * kCoreRow + 4 * e) = v.x;
-                    *reinterpret_cast<float *>(tab + l * kCoreRow + kCoreIm + 4 * e) = v.y;
-                }
+            stage_rows(tab, L.lut + gj * p * L.cmax1, p, L.cmax1, lane);
             if (GRAD)
                 for (int c = 0; c < 2 * p; ++c) sums[32 * c] = make_float2(0.f, 0.f);
         }
@@ -375,26 +272,12 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
                 }
             }
             // table entries of registers h and h + NP in the row of layer l
-            auto entry = [&](int h, int l) -> C2 {
-                const uint32_t row = tab0 + l * kCoreRow;
-                const uint32_t a = row + (__byte_perm(cnt[h >> 2], 0u, 0x4440u | uint32_t(h & 3)) << 1);
-                const uint32_t b = row + (__byte_perm(cnt[(h >> 2) + NW / 2], 0u, 0x4440u | uint32_t(h & 3)) << 1);
-                return C2{p2(lds1(a), lds1(b)), p2(lds1(a + kCoreIm), lds1(b + kCoreIm))};
-            };
-            auto weight = [&](int h) -> P2 {  // kCoreScale (c - c0)
-                return add2(p2(__uint_as_float(__byte_perm(cnt[h >> 2], 0x4B000000u, 0x7540u | uint32_t(h & 3))),
-                               __uint_as_float(
-                                   __byte_perm(cnt[(h >> 2) + NW / 2], 0x4B000000u, 0x7540u | uint32_t(h & 3)))),
-                            splat(-b0));
-            };
+            auto entry = [&](int h, int l) { return row_entry(tab0 + l * kCoreRow, cnt[h >> 2], cnt[(h >> 2) + NW / 2], h & 3); };
             float2 *__restrict__ sp = L.psi + it * block_amps + (u << T) + lane;
             C2 x[NP];
             if (L.load) {
 #pragma unroll
-                for (int h = 0; h < NP; ++h) {
-                    const float2 v = sp[h << 5], w = sp[(h + NP) << 5];
-                    x[h] = C2{p2(v.x, w.x), p2(v.y, w.y)};
-                }
+                for (int h = 0; h < NP; ++h) x[h] = load_pair(sp, h << 5, (h + NP) << 5);
             } else {
 #pragma unroll
                 for (int h = 0; h < NP; ++h) x[h] = entry(h, 0);
@@ -475,7 +358,7 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
                     float dg = 0.f, uw[NP], uv[NP];
 #pragma unroll
                     for (int h = 0; h < NP; ++h) {
-                        const float2 w = halves(weight(h)), v = halves(imconj(r[h], x[h]));
+                        const float2 w = halves(row_weight(cnt[h >> 2], cnt[(h >> 2) + NW / 2], h & 3, b0)), v = halves(imconj(r[h], x[h]));
                         dg = fmaf(w.x, v.x, dg);
                         uw[h] = w.y;
                         uv[h] = v.y;
@@ -509,11 +392,7 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
                 }
                 first_mix2<NP, true, true>(r, RB, 5, f1);
 #pragma unroll
-                for (int h = 0; h < NP; ++h) {
-                    const float2 a = halves(r[h].r), b = halves(r[h].i);
-                    sp[h << 5] = make_float2(a.x, b.x);
-                    sp[(h + NP) << 5] = make_float2(a.y, b.y);
-                }
+                for (int h = 0; h < NP; ++h) store_pair(sp, h << 5, (h + NP) << 5, r[h]);
             }
         }
         if (lane == 0) {
@@ -621,10 +500,7 @@ __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_ke
             if constexpr (MODE == kOuterFirst) {
                 C2 x[16];  // lambda
 #pragma unroll
-                for (int h = 0; h < 16; ++h) {
-                    const float2 u = sp[int64_t(h) << b], v = sp[int64_t(h + 16) << b];
-                    x[h] = C2{p2(u.x, v.x), p2(u.y, v.y)};
-                }
+                for (int h = 0; h < 16; ++h) x[h] = load_pair(sp, int64_t(h) << b, int64_t(h + 16) << b);
                 auto unmix = [&](auto form) {
 #pragma unroll
                     for (int q = 0; q < 5; ++q)
@@ -1126,15 +1002,6 @@ cudaError_t launch_split_wave(BigLaunch B, bool grad, int chunk_window, int64_t 
         win.push_back({w0, w0 + n, left > 5});
         w0 += n;
     }
-    // tiles per warp task (2^tile_bits tiles per item): as many as leave two tasks
-    // for every resident warp of 4 * blocks (of 1, 2, 4, 8, 16 tasks: 9.46, 8.77,
-    // 8.94, 9.02, 9.37 ms on the 6x6 torus at p = 3, energy, 32 points; within 3%
-    // for four cubic graphs n = 24, gradient)
-    auto tiles_per_task = [](int64_t items, int tile_bits, int blocks) {
-        int t = 1;
-        while (t < (1 << std::min(tile_bits, 6)) && (items << tile_bits) / (2 * t) >= int64_t(blocks) * 4 * 2) t *= 2;
-        return t;
-    };
     auto outer = [&](int mode, size_t w, int sign) -> cudaError_t {
         B.mode = mode;
         B.w0 = win[w].w0;

@@ -460,7 +460,6 @@ cudaError_t run_big(const qaoa_device_plan *d, const qaoa_plan *plan, int64_t P,
     cudaError_t e = launch_big_prep(params, int64_t(plan->n_graphs) * P, p, cs, fa, s);
     dm->all_launches += 1;
     const bool g = grad != nullptr;
-    const int grid = big_grid(g);
     for (const BigShape &bs : d->big) {
         if (e != cudaSuccess) break;
         const bool split = g ? bs.split_g : bs.split_e;
@@ -503,7 +502,7 @@ cudaError_t run_big(const qaoa_device_plan *d, const qaoa_plan *plan, int64_t P,
             }
             for (const BigPass &ps : passes) {
                 B.pass = ps;
-                e = launch_big_pass(B, g, grid, s);
+                e = launch_big_pass(B, g, s);
                 dm->all_launches += 1;
                 if (e != cudaSuccess) break;
             }

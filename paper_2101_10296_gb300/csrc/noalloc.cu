@@ -177,7 +177,6 @@ extern "C" int qaoa_energy_noalloc(const qaoa_plan *plan, int64_t n_points, cons
     // large-state cones: waves sized to the room left in the array
     if (e == cudaSuccess && !d->big.empty()) {
         e = launch_big_prep(params_dev, int64_t(GP), p, cs, nullptr, s);
-        const int grid = big_grid(false);
         int64_t launches = 0;
         for (const BigShape &bs : d->big) {
             if (e != cudaSuccess) break;
@@ -214,7 +213,7 @@ extern "C" int qaoa_energy_noalloc(const qaoa_plan *plan, int64_t n_points, cons
                 }
                 for (const BigPass &ps : bs.fwd) {
                     B.pass = ps;
-                    e = launch_big_pass(B, false, grid, s);
+                    e = launch_big_pass(B, false, s);
                     if (e != cudaSuccess) break;
                 }
             }
