@@ -187,7 +187,9 @@ inline size_t core_smem_bytes(int p, bool grad) { return size_t(4) * (p * kCoreR
 //
 // Bound: instruction fetch and latency (ncu, adjoint, p = 3: 49% of the issue
 // slots, FP32 pipe 52%, no-instruction the first stall; 5,000 instructions of
-// straight-line code), the energy by shuffles and shared memory (55%).  Measured
+// straight-line code, so that the block's warps start each tile together, which
+// lets them share fetched code: 14.4 -> 13.9 ms; further barriers within the tile or
+// larger blocks were slower), the energy by shuffles and shared memory (55%).  Measured
 // against the unpacked kernel with one tile per task: four cubic graphs n = 24,
 // p = 3, 25 points, gradient 21.6 -> 15.8 ms; 6x6 torus, p = 3, 32 points, energy
 // 10.1 -> 8.8 ms (both with their outer passes).
@@ -209,17 +211,18 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
     unsigned char *tab = s_core + warp * (p * kCoreRow);
     float2 *sums = reinterpret_cast<float2 *>(s_core + (blockDim.x >> 5) * (p * kCoreRow)) + warp * (2 * p * 32) + lane;
     const uint32_t tab0 = smem_addr(tab);
-    for (int64_t task = gw; task < ntask; task += nw) {
+    // the block's warps start every tile together (a warp past the last task, or of a
+    // foreign shape, only keeps step)
+    for (int64_t t0 = gw - warp; t0 < ntask; t0 += nw) {
+        const int64_t task = min(t0 + warp, ntask - 1);
         const int64_t it = task / per_item;
         const int64_t u0 = (task - it * per_item) * tpw;
         int ci;
         int64_t j, y;
         decode_item(L, L.item0 + it, ci, j, y);
         const DevCone *__restrict__ C = L.cones + L.cone_ids[ci];
-        if (__any_sync(kFull, C->n_in != nin)) {
-            if (lane == 0) atomicOr(L.status, 1);
-            continue;
-        }
+        const bool ours = t0 + warp < ntask && !__any_sync(kFull, C->n_in != nin);
+        if (t0 + warp < ntask && !ours && lane == 0) atomicOr(L.status, 1);
         const int64_t gj = int64_t(C->graph) * L.P + j;
         const float4 *__restrict__ cs = L.cs + gj * p;
         __syncwarp();
@@ -251,6 +254,8 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
         };
         Dfl e_sum{0.f, 0.f}, t_sum{0.f, 0.f};  // of the warp's tile sums
         for (int64_t u = u0; u < u0 + tpw; ++u) {
+            __syncthreads();
+            if (!ours) continue;
             uint64_t tb = base;
             for (int q = T; q < nin; ++q)
                 if ((u >> (q - T)) & 1) tb ^= C->col[q];
@@ -395,6 +400,7 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
                 for (int h = 0; h < NP; ++h) store_pair(sp, h << 5, (h + NP) << 5, r[h]);
             }
         }
+        if (!ours) continue;
         if (lane == 0) {
             atomicAdd(L.energy + gj, dfl_value(e_sum));
             if (L.terms) atomicAdd(L.terms + C->rep * L.P + j, dfl_value(t_sum));
