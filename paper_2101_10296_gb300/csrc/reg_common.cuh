@@ -58,7 +58,8 @@ __device__ __forceinline__ bool seg_sum(float &v, int key) {
 // (part, point): each lane adds G lanes' shares of its point with
 // compensation, the parts meet by shuffles, and lanes of part 0 add hi and lo
 // to the FP64 outputs of row row0 + point (row0 = g * n_points + first point
-// of the task) with separate atomics (no FP64 arithmetic).  Called by the
+// of the task), as one FP64 value (two atomics, one for each, took 0.38 against
+// 0.27 ms on a random cubic graph n = 1000, p = 2, 48 points, gradient).  Called by the
 // whole warp between __syncwarp()s.
 template <int UNROLL>
 __device__ __forceinline__ void reg_flush(const float *red, int nout, int G, int jj, int lane, int64_t row0,
@@ -79,8 +80,7 @@ __device__ __forceinline__ void reg_flush(const float *red, int nout, int G, int
         if (part == 0 && pt < gn) {
             const int64_t gjj = row0 + jf + pt;
             double *dst = c == 0 ? energy + gjj : grad + gjj * n_grad + (c - 1);
-            atomicAdd(dst, f2d(acc.hi));
-            if (acc.lo != 0.f) atomicAdd(dst, f2d(acc.lo));
+            atomicAdd(dst, f2d(acc.hi) + f2d(acc.lo));  // one addition: the outputs of a point are contended
         }
     }
 }
