@@ -91,6 +91,33 @@ __device__ __forceinline__ void store_amp(float2 *p, P2 v) { *reinterpret_cast<u
 // Cut words as 32 bits where every cone of the plan fits them, else 64.
 __device__ __forceinline__ int popc_w(uint32_t x) { return __popc(x); }
 __device__ __forceinline__ int popc_w(uint64_t x) { return __popcll(x); }
+// Scaled cut values over G window bits.  With the fixed bits' word base, setting
+// bit q adds d_q = popc(base ^ col_q) - popc(base), and setting q and q' together
+// adds pair_qq' more, -2 for each positive (+2 for each negative) cut bit of an
+// edge that joins them, whatever base is: so a lane counts G + 1 words and adds up
+// the others (two integer additions per value instead of a 64-bit exclusive or, two
+// popcounts and an addition).  The pairs are uniform: pairs[q (q - 1) / 2 + q'].
+constexpr int kPairs5 = 10;
+template <typename MT>
+__device__ __forceinline__ int window_pair(MT a, MT b, MT neg) {
+    return 2 * (popc_w(MT(a & b & neg)) - popc_w(MT(a & b & ~neg)));
+}
+template <int G, int SCALE, typename MT>
+__device__ __forceinline__ void window_counts(MT base, const MT (&col)[5], const int (&pairs)[kPairs5], int (&c)[1 << G]) {
+    const int n = popc_w(base);
+    c[0] = SCALE * n;
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+        int e[1 << (G - 1)];
+        e[0] = SCALE * (popc_w(MT(base ^ col[q])) - n);
+#pragma unroll
+        for (int i = 0; i < (1 << q); ++i) {
+            const int t = i < 2 ? 0 : i < 4 ? 1 : i < 8 ? 2 : 3;  // the highest bit of i > 0
+            if (i > 0) e[i] = e[i ^ (1 << t)] + SCALE * pairs[q * (q - 1) / 2 + t];
+            c[i | (1 << q)] = c[i] + e[i];
+        }
+    }
+}
 // XOR over the lanes.
 __device__ __forceinline__ uint32_t warp_xor(uint32_t x) { return __reduce_xor_sync(kFull, x); }
 __device__ __forceinline__ uint64_t warp_xor(uint64_t x) {

@@ -466,7 +466,8 @@ __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_ke
         const int64_t gj = int64_t(C->graph) * L.P + j;
         const FirstMix f1 = first_mix(L, gj, nin);
         float mult = 1.f;
-        MT item_w = 0, bit_w = 0, lo[4], wh[8];
+        MT item_w = 0, bit_w = 0, col[5];
+        int pairs[kPairs5];
         if (MODE != kOuterMix) {
             // first layer's phase table: entries (kOuterGen), or real parts, then imaginary parts
             __syncwarp();
@@ -486,15 +487,12 @@ __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_ke
             for (int lb = 0; lb < 5; ++lb)
                 if ((lane >> lb) & 1) item_w ^= MT(C->col[RB + lb]);
             if (lane >= 5 && lane < nin && (lane < b || lane >= b + 5)) bit_w = MT(C->col[qubit_of(lane, RB)]);
-            const MT c0 = MT(C->col[qubit_of(b, RB)]), c1 = MT(C->col[qubit_of(b + 1, RB)]);
-            const MT c2 = MT(C->col[qubit_of(b + 2, RB)]), c3 = MT(C->col[qubit_of(b + 3, RB)]);
-            const MT c4 = MT(C->col[qubit_of(b + 4, RB)]);
-            lo[0] = 0;
-            lo[1] = c0;
-            lo[2] = c1;
-            lo[3] = c0 ^ c1;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) wh[k] = ((k & 1) ? c2 : MT(0)) ^ ((k & 2) ? c3 : MT(0)) ^ ((k & 4) ? c4 : MT(0));
+            for (int q = 0; q < 5; ++q) col[q] = MT(C->col[qubit_of(b + q, RB)]);
+#pragma unroll
+            for (int q = 1; q < 5; ++q)
+#pragma unroll
+                for (int t = 0; t < q; ++t) pairs[q * (q - 1) / 2 + t] = uniform(window_pair(col[q], col[t], MT(C->neg)));
         }
         Dfl s_dg{0.f, 0.f}, s_db{0.f, 0.f};
         for (int64_t tile = tile0; tile < tile0 + tpw; ++tile) {
@@ -525,17 +523,14 @@ __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_ke
                 const float b0 = 4194304.f + 0.5f * float(C->m);  // Im<lambda|psi> = 0: C - c0 in place of C
                 const float *tr = s_tab[warp], *ti = s_tab[warp] + kOuterRow;
                 // state before the first mixer, times 2^(n/2), of registers h and h + 16
-                auto phase = [&](MT w, int h, int &cl, int &cu) -> C2 {
-                    cl = popc_w(MT(lo[h & 3] ^ wh[h >> 2] ^ w));
-                    cu = popc_w(MT(lo[h & 3] ^ wh[(h >> 2) + 4] ^ w));
-                    return C2{p2(tr[cl], tr[cu]), p2(ti[cl], ti[cu])};
-                };
+                int cnt[32];
+                window_counts<5, 1>(base, col, pairs, cnt);
                 C2 ph[16];
                 float dg = 0.f, uw[16], uv[16];
 #pragma unroll
                 for (int h = 0; h < 16; ++h) {
-                    int cl, cu;
-                    ph[h] = phase(base, h, cl, cu);
+                    const int cl = cnt[h], cu = cnt[h + 16];
+                    ph[h] = C2{p2(tr[cl], tr[cu]), p2(ti[cl], ti[cu])};
                     const float2 v = halves(imconj(x[h], ph[h]));
                     dg = fmaf(cut_minus(cl, b0), v.x, dg);
                     uw[h] = cut_minus(cu, b0);
@@ -562,12 +557,13 @@ __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_ke
                         dfl_add(db, d);
                     }
                     for (int q = L.x0; q < L.x1; ++q) {  // outer qubits outside the window
-                        const MT w = base ^ MT(C->col[q]);
+                        // (qubit q's edges into the window shift its counts: the sums start over)
+                        window_counts<5, 1>(MT(base ^ MT(C->col[q])), col, pairs, cnt);
                         float t = 0.f;
 #pragma unroll
                         for (int h = 0; h < 16; ++h) {
-                            int cl, cu;
-                            const float2 v = halves(imconj(x[h], phase(w, h, cl, cu)));
+                            const int cl = cnt[h], cu = cnt[h + 16];
+                            const float2 v = halves(imconj(x[h], C2{p2(tr[cl], tr[cu]), p2(ti[cl], ti[cu])}));
                             t += v.x;
                             uv[h] = v.y;
                         }
@@ -581,8 +577,10 @@ __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_ke
                 P2 x[32];
                 if (MODE == kOuterGen) {
                     const float2 *tab = reinterpret_cast<const float2 *>(s_tab[warp]);
+                    int cnt[32];
+                    window_counts<5, 1>(base, col, pairs, cnt);
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) x[i] = load_amp(tab + popc_w(MT(lo[i & 3] ^ wh[i >> 2] ^ base)));
+                    for (int i = 0; i < 32; ++i) x[i] = load_amp(tab + cnt[i]);
                     first_mix_regs<32, false, LO>(x, r0, r1, f1);
                 } else {
 #pragma unroll
@@ -701,32 +699,37 @@ template <typename MT>
 struct ChunkItem {
     float2 tab[kOuterRow];
     MT col[kChunkBits];
+    int pairs[kPairs5];  // of the first round's window bits (see window_counts)
 };
 
-// First-layer cut words over the G register bits from chunk bit pos on: lo over
-// the first two, hi over the rest, with the slot's fixed bits sb and cw.
+// First-layer cut values over the G register bits from chunk bit pos on (the
+// window's lowest), with the slot's fixed bits sb and cw.
 template <int G, typename MT>
-__device__ __forceinline__ void slot_words(const ChunkItem<MT> &I, MT cw, int sb, int pos, MT (&lo)[4], MT (&hi)[8]) {
+__device__ __forceinline__ void slot_counts(const ChunkItem<MT> &I, MT cw, int sb, int pos, int (&c)[1 << G]) {
     MT base = cw;
 #pragma unroll
     for (int b = 0; b < kChunkBits; ++b)
         if ((sb >> b) & 1) base ^= I.col[b];  // the register bits of sb are zero
-    MT cr[5];
+    MT col[5];
+    int pairs[kPairs5];
 #pragma unroll
-    for (int b = 0; b < 5; ++b) cr[b] = b < G ? I.col[pos + b] : MT(0);
-    lo[0] = 0;
-    lo[1] = cr[0];
-    lo[2] = cr[1];
-    lo[3] = cr[0] ^ cr[1];
+    for (int b = 0; b < 5; ++b) col[b] = b < G ? I.col[pos + b] : MT(0);
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-        hi[k] = base ^ ((k & 1) ? cr[2] : MT(0)) ^ ((k & 2) ? cr[3] : MT(0)) ^ ((k & 4) ? cr[4] : MT(0));
+    for (int k = 0; k < kPairs5; ++k) pairs[k] = I.pairs[k];
+    window_counts<G, 1>(base, col, pairs, c);
+}
+
+// A chunk element's place: the swizzled one where asked for (SW: the chunk's
+// geometry has a swizzle at all).
+template <bool SW>
+__device__ __forceinline__ int place(int s, bool swizzled) {
+    return SW ? sidx(s, swizzled) : s;
 }
 
 // One round of a chunk pass: every slot gathers the 2^G amplitudes that
 // differ in chunk bits [pos, pos+G), applies the mixer to those G qubits and
 // writes them back.  GEN in its first round generates the amplitudes instead.
-template <int G, bool GEN, bool INV, bool LO, typename MT>
+template <int G, bool GEN, bool INV, bool LO, bool SW, typename MT>
 __device__ __forceinline__ void chunk_round(float2 *__restrict__ sm, int n_el, int pos, const FirstMix &f,
                                             const ChunkItem<MT> &I, MT cw, bool rd_swz, bool wr_swz) {
     constexpr int NR = 1 << G;
@@ -734,30 +737,43 @@ __device__ __forceinline__ void chunk_round(float2 *__restrict__ sm, int n_el, i
         const int sb = spread_slot(slot, pos, G);
         P2 x[NR];
         if (GEN) {
-            MT lo[4], hi[8];
-            slot_words<G>(I, cw, sb, pos, lo, hi);
+            int c[NR];
+            slot_counts<G>(I, cw, sb, pos, c);
 #pragma unroll
-            for (int i = 0; i < NR; ++i) x[i] = load_amp(I.tab + popc_w(MT(lo[i & 3] ^ hi[i >> 2])));
+            for (int i = 0; i < NR; ++i) x[i] = load_amp(I.tab + c[i]);
         } else {
 #pragma unroll
-            for (int i = 0; i < NR; ++i) x[i] = load_amp(sm + sidx(sb | (i << pos), rd_swz));
+            for (int i = 0; i < NR; ++i) x[i] = load_amp(sm + place<SW>(sb + (i << pos), rd_swz));
         }
         first_mix_regs<NR, INV, LO>(x, 0, G, f);
 #pragma unroll
-        for (int i = 0; i < NR; ++i) store_amp(sm + sidx(sb | (i << pos), wr_swz), x[i]);
+        for (int i = 0; i < NR; ++i) store_amp(sm + place<SW>(sb + (i << pos), wr_swz), x[i]);
     }
 }
 
+template <bool GEN, bool INV, bool LO, bool SW, typename MT>
+__device__ __forceinline__ void chunk_round_g(int G, float2 *sm, int n_el, int pos, const FirstMix &f,
+                                              const ChunkItem<MT> &I, MT cw, bool rd_swz, bool wr_swz) {
+    switch (G) {
+        case 1: chunk_round<1, GEN, INV, LO, SW>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
+        case 2: chunk_round<2, GEN, INV, LO, SW>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
+        case 3: chunk_round<3, GEN, INV, LO, SW>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
+        case 4: chunk_round<4, GEN, INV, LO, SW>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
+        default: chunk_round<5, GEN, INV, LO, SW>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
+    }
+}
+
+// sw: the chunk's runs are short enough (eight amplitudes, a window of ten, whose
+// rounds all have five bits) for the swizzle.  A first round always has five.
 template <bool GEN, bool INV, bool LO, typename MT>
 __device__ __forceinline__ void chunk_round_any(int G, float2 *sm, int n_el, int pos, const FirstMix &f,
-                                                const ChunkItem<MT> &I, MT cw, bool rd_swz, bool wr_swz) {
-    switch (G) {
-        case 1: chunk_round<1, GEN, INV, LO>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
-        case 2: chunk_round<2, GEN, INV, LO>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
-        case 3: chunk_round<3, GEN, INV, LO>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
-        case 4: chunk_round<4, GEN, INV, LO>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
-        default: chunk_round<5, GEN, INV, LO>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz); break;
-    }
+                                                const ChunkItem<MT> &I, MT cw, bool sw, bool rd_swz, bool wr_swz) {
+    if (sw)
+        chunk_round<5, GEN, INV, LO, true>(sm, n_el, pos, f, I, cw, rd_swz, wr_swz);
+    else if (GEN)
+        chunk_round<5, GEN, INV, LO, false>(sm, n_el, pos, f, I, cw, false, false);
+    else
+        chunk_round_g<GEN, INV, LO, false>(G, sm, n_el, pos, f, I, cw, false, false);
 }
 
 template <int MODE, bool LO, typename MT>
@@ -808,6 +824,10 @@ __global__ void __launch_bounds__(kChunkThreads, 2)
             for (int e = tid; e < L.cmax1; e += kChunkThreads) s_item.tab[e] = __ldg(lut + e);
             if (tid < kChunkBits)
                 s_item.col[tid] = MT(C->col[tid < lo_bits ? qubit_of(tid, RB) : w0 + tid - lo_bits]);
+            if (tid < kPairs5) {  // pair (q, t), t < q
+                const int q = tid < 1 ? 1 : tid < 3 ? 2 : tid < 6 ? 3 : 4, t = tid - q * (q - 1) / 2;
+                s_item.pairs[tid] = window_pair(MT(C->col[w0 + q]), MT(C->col[w0 + t]), MT(C->neg));
+            }
             cw = MT(shell_block(C, L.shell, uint32_t(y), mult));
             for (int a = lo_bits; a < nin; ++a)
                 if ((a < w0 || a >= w0 + w) && ((xb >> a) & 1)) cw ^= MT(C->col[qubit_of(a, RB)]);
@@ -830,11 +850,11 @@ __global__ void __launch_bounds__(kChunkThreads, 2)
             const bool swz_on = lo_bits < 4;
             const bool rd_swz = swz_on && g0 > 0, wr_swz = swz_on && (g0 + gn < w || MODE == kOuterFirst);
             if (MODE == kOuterGen && g0 == 0)
-                chunk_round_any<true, false, LO>(gn, sm, n_el, lo_bits, f1, s_item, cw, rd_swz, wr_swz);
+                chunk_round_any<true, false, LO>(gn, sm, n_el, lo_bits, f1, s_item, cw, swz_on, rd_swz, wr_swz);
             else if (MODE == kOuterGen || (MODE == kOuterMix && L.sign > 0))
-                chunk_round_any<false, false, LO>(gn, sm, n_el, lo_bits + g0, f1, s_item, cw, rd_swz, wr_swz);
+                chunk_round_any<false, false, LO>(gn, sm, n_el, lo_bits + g0, f1, s_item, cw, swz_on, rd_swz, wr_swz);
             else
-                chunk_round_any<false, true, LO>(gn, sm, n_el, lo_bits + g0, f1, s_item, cw, rd_swz, wr_swz);
+                chunk_round_any<false, true, LO>(gn, sm, n_el, lo_bits + g0, f1, s_item, cw, swz_on, rd_swz, wr_swz);
             __syncthreads();
         }
         if (MODE == kOuterFirst) {
@@ -851,12 +871,12 @@ __global__ void __launch_bounds__(kChunkThreads, 2)
 #pragma unroll
                 for (int i = 0; i < 32; ++i)
                     x[i] = i < nreg ? sm[sidx(sb | (i << lo_bits), lo_bits < 4)] : make_float2(0.f, 0.f);
-                MT lo[4], hi[8];
-                slot_words<5>(s_item, cw, sb, lo_bits, lo, hi);  // w > 5 here: five window qubits in registers
+                int cnt[32];
+                slot_counts<5>(s_item, cw, sb, lo_bits, cnt);  // w > 5 here: five window qubits in registers
                 float dgs = 0.f, dq[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
-                    const int c = popc_w(MT(lo[i & 3] ^ hi[i >> 2]));
+                    const int c = cnt[i];
                     const float2 ph = s_item.tab[c];
                     dgs = fmaf(cut_minus(c, b0), imconj(x[i], ph), dgs);
                     if (outer_terms) {
@@ -870,11 +890,10 @@ __global__ void __launch_bounds__(kChunkThreads, 2)
                     for (int rb = 0; rb < 5; ++rb) dfl_add(db, dq[rb]);
                     // the other outer qubits: the rest of the window, then beyond it
                     for (int q = w0 + 5; q < L.x1; ++q) {
-                        const MT cq = MT(C->col[q]);
+                        slot_counts<5>(s_item, MT(cw ^ MT(C->col[q])), sb, lo_bits, cnt);
                         float t = 0.f;
 #pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            t += imconj(x[i], s_item.tab[popc_w(MT(lo[i & 3] ^ hi[i >> 2] ^ cq))]);
+                        for (int i = 0; i < 32; ++i) t += imconj(x[i], s_item.tab[cnt[i]]);
                         dfl_add(db, t);
                     }
                 }
