@@ -79,7 +79,6 @@ struct BigLaunch {
 // cone, point by point, shell block by shell block.
 std::vector<BigPass> big_forward_passes(int n_in, int p, const int32_t *k);
 std::vector<BigPass> big_grad_passes(int n_in, int p, const int32_t *k);
-cudaError_t launch_big_prep(const double *params, int64_t GP, int p, float4 *cs, float2 *fa, cudaStream_t s);
 cudaError_t launch_big_pass(BigLaunch a, bool grad, cudaStream_t s);
 // Tiles per warp task (2^tile_bits tiles per item): as many as leave two tasks
 // for every resident warp of 4 * blocks (of 1, 2, 4, 8, 16 tasks: 9.46, 8.77,

@@ -484,13 +484,12 @@ namespace {
 
 // Large-state cones: per shape, waves of blocks that fit the scratch budget,
 // each wave streamed through the shape's pass list.
-cudaError_t run_big(const qaoa_device_plan *d, const qaoa_plan *plan, int64_t P, const double *params,
-                    const float2 *lut, const float2 *mix, const float *kpow, double *energy, double *grad,
+cudaError_t run_big(const qaoa_device_plan *d, const qaoa_plan *plan, int64_t P, const float2 *lut,
+                    const float2 *mix, const float *kpow, double *energy, double *grad,
                     double *terms, bool norm, float4 *cs, float2 *fa, cudaStream_t s) {
     qaoa_device_plan *dm = const_cast<qaoa_device_plan *>(d);
     const int p = plan->p;
-    cudaError_t e = launch_big_prep(params, int64_t(plan->n_graphs) * P, p, cs, fa, s);
-    dm->all_launches += 1;
+    cudaError_t e = cudaSuccess;
     const bool g = grad != nullptr;
     for (const BigShape &bs : d->big) {
         if (e != cudaSuccess) break;
@@ -589,6 +588,8 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
     pa.terms = terms;
     pa.n_reps = d->n_cones;
     pa.n_kpow = d->n_kpow;
+    pa.cs = cs;
+    pa.fa = fa;
     e = launch_prep(pa, s);
     qaoa_device_plan *dm = const_cast<qaoa_device_plan *>(d);
     dm->all_launches += 1;
@@ -639,7 +640,7 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
         int64_t grid = std::min<int64_t>(tuned_grid(d, reg_p1_grid(grad != nullptr, d->cmax1, smem)), (tasks + 3) / 4);
         e = launch_reg_p1(L, grad != nullptr, int(std::max<int64_t>(grid, 1)), s);
         dm->all_launches += 1;
-        if (e == cudaSuccess && !d->big.empty()) e = run_big(d, plan, n_points, params, lut, mix, kpow, energy, grad, terms, norm, cs, fa, s);
+        if (e == cudaSuccess && !d->big.empty()) e = run_big(d, plan, n_points, lut, mix, kpow, energy, grad, terms, norm, cs, fa, s);
     } else if (e == cudaSuccess) {
         RegLaunch L;
         L.n_points = n_points;
@@ -658,7 +659,7 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
         L.work = as_reg(d, d->reg[rg - 4]);
         if (L.work.warps > 0) e = launch_reg(d, L, g, rg, d->points_per_task, s);
         if (L.work.warps > 0) dm->all_launches += 1;
-        if (e == cudaSuccess && !d->big.empty()) e = run_big(d, plan, n_points, params, lut, mix, kpow, energy, grad, terms, norm, cs, fa, s);
+        if (e == cudaSuccess && !d->big.empty()) e = run_big(d, plan, n_points, lut, mix, kpow, energy, grad, terms, norm, cs, fa, s);
     }
     if (ev0) {
         cudaEventRecord(ev1, s);

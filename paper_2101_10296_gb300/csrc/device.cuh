@@ -140,6 +140,8 @@ struct PrepArgs {
     double *terms;            // may be null
     int64_t n_reps;
     int32_t n_kpow;           // kappa powers filled per row: what the plan's mixers read (<= kKpow)
+    float4 *cs;               // large-state cones: exact rotations [G][P][p]; null: none
+    float2 *fa;               // their first layer's factored coefficient, hi and lo [G][P]; may be null
 };
 
 // launchers (kernels.cu)

@@ -51,6 +51,8 @@ namespace {
 // Measured: the whole call of an 8x8 torus at p = 2, 128 points, energy 35 -> 17
 // us (256 rows of 24 entries had sat on one SM, 33 kappa powers each where 10
 // are read); the 48-graph mix at p = 1, 256 points 763 -> 749 us.
+// The large-state kernels' rotations come from the same sincos (a launch of their
+// own before: 59.1 -> 56.8 us for the 5x5 torus, p = 3, 4 points, energy).
 constexpr int kPrepBlock = 64;
 
 __global__ void __launch_bounds__(kPrepBlock) prep_kernel(const PrepArgs a, int parts, int row_blocks, int mix_blocks) {
@@ -98,6 +100,22 @@ __global__ void __launch_bounds__(kPrepBlock) prep_kernel(const PrepArgs a, int 
         for (int k = 0; k < a.n_kpow; ++k) {
             a.kpow[u * kKpow + k] = float(pw);
             pw *= k2;
+        }
+        // (cos beta, sin beta) for the large-state kernels' exact rotations, each as an FP32 pair hi + lo.
+        // Rounded to one FP32 number each, the gate becomes r exp(-i beta' X) with beta' - beta up to
+        // ~4e-8: the same shift for every amplitude, layer after layer, which a small gradient (near a
+        // stationary point, a second derivative times that shift) feels in full.  The lo parts (two more
+        // FMAs per output) take the shift away; what remains is per-operation rounding.
+        if (a.cs) {
+            const float ch = float(cs), sh = float(sn);
+            a.cs[u] = make_float4(ch, sh, float(cs - double(ch)), float(sn - double(sh)));
+        }
+        if (a.fa && l == 0) {
+            // the first layer's factored coefficient: tan beta, or cot beta where |tan beta| > 1 (tau's
+            // choice and rounded hi part, but for the sign), with its FP32 rounding error
+            const double f = flip ? cs / sn : sn / cs;
+            const float fh = float(f);
+            a.fa[gj] = make_float2(fh, float(f - double(fh)));
         }
         return;
     }

@@ -135,6 +135,8 @@ extern "C" int qaoa_energy_noalloc(const qaoa_plan *plan, int64_t n_points, cons
     pa.terms = terms_dev;
     pa.n_reps = d->n_cones;
     pa.n_kpow = d->n_kpow;
+    pa.cs = d->big.empty() ? nullptr : cs;
+    pa.fa = nullptr;
     e = launch_prep(pa, s);
     // register-resident cones: the depth-1 kernel where the plan has its list
     // (p = 1, no per-cone terms asked for), else the general register kernel
@@ -176,7 +178,6 @@ extern "C" int qaoa_energy_noalloc(const qaoa_plan *plan, int64_t n_points, cons
     }
     // large-state cones: waves sized to the room left in the array
     if (e == cudaSuccess && !d->big.empty()) {
-        e = launch_big_prep(params_dev, int64_t(GP), p, cs, nullptr, s);
         int64_t launches = 0;
         for (const BigShape &bs : d->big) {
             if (e != cudaSuccess) break;
