@@ -33,7 +33,7 @@ constexpr int NW = 8;                       // packed cut counts, 4 registers pe
 // 1.24 ms, energy 0.50 -> 0.30 ms.
 template <bool GRAD, typename MT>
 __global__ void __launch_bounds__(128) big_pass_kernel(const __grid_constant__ BigLaunch L) {
-    chain_wait();
+    wait_before();
     extern __shared__ __align__(256) unsigned char s_big[];
     const int lane = threadIdx.x & 31, warp = warp_index();
     const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp;
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(128) big_pass_kernel(const __grid_constant__ B
 // No cut words or tables, so far fewer registers and more loads in flight.  An
 // amplitude per packed register.
 __global__ void __launch_bounds__(128, 4) big_mix_kernel(const __grid_constant__ BigLaunch L) {
-    chain_wait();
+    wait_before();
     constexpr int NR = 2 * NP;
     const int lane = threadIdx.x & 31;
     const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp_index();
@@ -328,20 +328,6 @@ const void *pass_fn(bool grad, bool wide) {
 
 }  // namespace
 
-cudaError_t launch_chain(const void *fn, const BigLaunch &L, int grid, int block, void **args, size_t smem, cudaStream_t s) {
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c{};
-    c.gridDim = dim3(unsigned(grid));
-    c.blockDim = dim3(unsigned(block));
-    c.dynamicSmemBytes = smem;
-    c.stream = s;
-    c.attrs = &attr;
-    c.numAttrs = L.chained ? 1 : 0;
-    return cudaLaunchKernelExC(&c, fn, args);
-}
-
 static bool mix_only(const BigPass &ps) {
     if (!ps.load_psi || !ps.store_psi || ps.load_lam || ps.store_lam) return false;
     for (int o = 0; o < ps.nops; ++o)
@@ -355,7 +341,7 @@ cudaError_t launch_big_pass(BigLaunch a, bool grad, cudaStream_t s) {
     if (mix_only(a.pass)) {
         const int64_t need = std::max<int64_t>(1, (tiles + 3) / 4);
         void *args[] = {&a};
-        return launch_chain((const void *)big_mix_kernel, a, int(std::min<int64_t>(mix_grid(), need)), 128, args, 0, s);
+        return launch_after((const void *)big_mix_kernel, int(std::min<int64_t>(mix_grid(), need)), 128, args, 0, s);
     }
     const size_t smem = size_t(4) * (a.p * kCoreRow + (grad ? 2 * a.p * 32 * sizeof(float2) : 0));
     const void *fn = pass_fn(grad, a.cmax1 - 1 > 32);
@@ -363,7 +349,7 @@ cudaError_t launch_big_pass(BigLaunch a, bool grad, cudaStream_t s) {
     a.tpw = tiles_per_task(a.n_items, bits, full);
     const int64_t need = std::max<int64_t>(1, (tiles / a.tpw + 3) / 4);
     void *args[] = {&a};
-    return launch_chain(fn, a, int(std::min<int64_t>(full, need)), 128, args, smem, s);
+    return launch_after(fn, int(std::min<int64_t>(full, need)), 128, args, smem, s);
 }
 
 // ------------------------------------------------------------ pass lists

@@ -73,7 +73,6 @@ struct BigLaunch {
     int32_t mode, sign;       // SplitOuterMode; +1 mix, -1 un-mix (kOuterMix)
     int32_t load;             // core pass: load the tile (1) or generate layer 1's phase state (0)
     int32_t tpw;              // consecutive tiles of an item per warp task (a power of two)
-    int32_t chained;          // the launch before it in the stream is of the same chain (host side)
 };
 
 // Cones of one shape share n_in and k; items of a wave are numbered cone by
@@ -81,13 +80,6 @@ struct BigLaunch {
 std::vector<BigPass> big_forward_passes(int n_in, int p, const int32_t *k);
 std::vector<BigPass> big_grad_passes(int n_in, int p, const int32_t *k);
 cudaError_t launch_big_pass(BigLaunch a, bool grad, cudaStream_t s);
-// One launch of a chain (the passes over one shape's blocks): where L.chained, it is
-// prepared while the launch before it drains (programmatic stream serialisation), and
-// its kernel begins with chain_wait().  The first launch of a chain is a plain one:
-// an allocation stands before it.  Between small passes the launches' own latency
-// counts: cubic n = 16, p = 3, 14 points, energy 125 -> 115 us; n = 20, 4 points,
-// gradient 375 -> 348; circulant n = 30, p = 4, 64 points, gradient 1233 -> 1217.
-cudaError_t launch_chain(const void *fn, const BigLaunch &L, int grid, int block, void **args, size_t smem, cudaStream_t s);
 // Tiles per warp task (2^tile_bits tiles per item): as many as leave two tasks
 // for every resident warp of 4 * blocks (of 1, 2, 4, 8, 16 tasks: 9.46, 8.77,
 // 8.94, 9.02, 9.37 ms on the 6x6 torus at p = 3, energy, 32 points; within 3%

@@ -8,15 +8,6 @@
 namespace qaoa {
 namespace {
 
-// Start of a chain's kernel, run by every thread before any access to memory: waits
-// until the launch before has ended and its writes are visible (at once where the
-// launch was a plain one).  The next launch is let in when this one's blocks end;
-// letting it in from the start as well cost the passes 3-11% (four cubic graphs n =
-// 24: 13.7 -> 14.6 ms).
-__device__ __forceinline__ void chain_wait() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
 // One output of exp(-i beta X) on the pair (me, o), c me - i s o, or of
 // exp(+i beta X) (INV), with c = cs.x + cs.z and s = cs.y + cs.w (hi and lo FP32
 // parts), on the amplitudes of two packed registers.

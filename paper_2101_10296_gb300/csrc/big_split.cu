@@ -195,7 +195,7 @@ inline size_t core_smem_bytes(int p, bool grad) { return size_t(4) * (p * kCoreR
 // 10.1 -> 8.8 ms (both with their outer passes).
 template <bool GRAD, int RB>
 __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlocks) split_core_kernel(const __grid_constant__ BigLaunch L) {
-    chain_wait();
+    wait_before();
     constexpr int NR = 1 << RB, NP = NR / 2;
     constexpr int T = RB + 5;
     constexpr int NW = NR / 4;  // packed cut counts, 4 registers per word
@@ -441,7 +441,7 @@ __device__ __forceinline__ int qubit_of(int a, int rb) { return a < 5 ? rb + a :
 // energy 8.8 -> 8.3 ms; Q_12 full cone, 32 points, energy 4.5 -> 4.15 ms.
 template <int MODE, bool LO, typename MT>
 __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_kernel(const __grid_constant__ BigLaunch L) {
-    chain_wait();
+    wait_before();
     __shared__ __align__(16) float s_tab[4][MODE == kOuterMix ? 4 : 2 * kOuterRow];
     const int lane = threadIdx.x & 31, warp = warp_index();
     const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp;
@@ -781,7 +781,7 @@ __device__ __forceinline__ void chunk_round_any(int G, float2 *sm, int n_el, int
 template <int MODE, bool LO, typename MT>
 __global__ void __launch_bounds__(kChunkThreads, 2)
     split_chunk_kernel(const __grid_constant__ BigLaunch L, const __grid_constant__ CUtensorMap tmap) {
-    chain_wait();
+    wait_before();
     extern __shared__ __align__(1024) float2 sm[];
     __shared__ uint64_t s_bar;  // completion of the chunk's load
     __shared__ ChunkItem<MT> s_item;
@@ -1046,7 +1046,7 @@ cudaError_t launch_split_wave(BigLaunch B, bool grad, int chunk_window, int64_t 
             const void *fn = chunk_fn(mode, grad, wide);
             const int grid = int(std::min<int64_t>(occupancy_grid(fn, kChunkThreads, kChunkSmem), std::max<int64_t>(tasks, 1)));
             void *args[] = {&B, &map};
-            if (cudaError_t e = launch_chain(fn, B, grid, kChunkThreads, args, kChunkSmem, s); e != cudaSuccess) return e;
+            if (cudaError_t e = launch_after(fn, grid, kChunkThreads, args, kChunkSmem, s); e != cudaSuccess) return e;
         } else {
             const void *fn = outer_fn(mode, grad, wide);
             const int full = occupancy_grid(fn, 128, 0);
@@ -1054,10 +1054,9 @@ cudaError_t launch_split_wave(BigLaunch B, bool grad, int chunk_window, int64_t 
             const int64_t tasks = (B.n_items << (nin - 10)) / B.tpw;
             const int grid = int(std::min<int64_t>(full, std::max<int64_t>(1, (tasks + 3) / 4)));
             void *args[] = {&B};
-            if (cudaError_t e = launch_chain(fn, B, grid, 128, args, 0, s); e != cudaSuccess) return e;
+            if (cudaError_t e = launch_after(fn, grid, 128, args, 0, s); e != cudaSuccess) return e;
         }
         ++launches;
-        B.chained = 1;
         return cudaSuccess;
     };
     if (grad && win.empty()) return cudaErrorInvalidValue;  // excluded by split_ok
@@ -1073,9 +1072,8 @@ cudaError_t launch_split_wave(BigLaunch B, bool grad, int chunk_window, int64_t 
     const int64_t core_tasks = (B.n_items << (nin - T)) / B.tpw;
     const int grid = int(std::min<int64_t>(core_grid, std::max<int64_t>(1, (core_tasks + 3) / 4)));
     void *args[] = {&B};
-    if ((e = launch_chain(core, B, grid, 128, args, core_smem, s)) != cudaSuccess) return e;
+    if ((e = launch_after(core, grid, 128, args, core_smem, s)) != cudaSuccess) return e;
     ++launches;
-    B.chained = 1;
     if (!grad) return cudaSuccess;
     for (size_t w = win.size(); w-- > 1 && e == cudaSuccess;) e = outer(kOuterMix, w, -1);
     if (e != cudaSuccess) return e;

@@ -529,13 +529,11 @@ cudaError_t run_big(const qaoa_device_plan *d, const qaoa_plan *plan, int64_t P,
             B.n_items = std::min(wave, items - i0);
             if (split) {
                 e = launch_split_wave(B, g, d->chunk_window, dm->all_launches, s);
-                B.chained = 1;
                 continue;
             }
             for (const BigPass &ps : passes) {
                 B.pass = ps;
                 e = launch_big_pass(B, g, s);
-                B.chained = 1;
                 dm->all_launches += 1;
                 if (e != cudaSuccess) break;
             }

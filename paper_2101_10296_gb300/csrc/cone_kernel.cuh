@@ -215,6 +215,7 @@ constexpr int kFlushUnroll = QAOA_FLUSH_UNROLL;
 template <int R, typename MT, bool GRAD, int PC>
 __global__ void __launch_bounds__(kRegBlock, GRAD ? (R <= 4 ? kGradMinBlocks : kGradMinBlocks5) : kEnergyMinBlocks)
     reg_cone_kernel(const RegLaunch L) {
+    wait_before();
     constexpr int NA = 1 << R;
     extern __shared__ float2 s_tab[];
     const int lane = threadIdx.x & 31;

@@ -26,11 +26,9 @@ cudaError_t depth2_prepare_r() {
 template <int R, bool GRAD>
 cudaError_t launch_depth2_r(const RegLaunch &a, int grid, cudaStream_t s) {
     const size_t sm = depth2_smem_bytes(a.jpt, a.cmax1, GRAD);
-    if (depth2_narrow(a.cmax1))
-        depth2_kernel<R, GRAD, true><<<grid, kRegBlock, sm, s>>>(a);
-    else
-        depth2_kernel<R, GRAD, false><<<grid, kRegBlock, sm, s>>>(a);
-    return cudaGetLastError();
+    RegLaunch arg = a;
+    void *args[] = {&arg};
+    return launch_after(depth2_fn_r<R, GRAD>(a.cmax1), grid, kRegBlock, args, sm, s);
 }
 
 }  // namespace qaoa

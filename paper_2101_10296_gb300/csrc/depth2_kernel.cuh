@@ -103,6 +103,7 @@ __device__ __forceinline__ void opaque(uint32_t &v) { asm volatile("" : "+r"(v))
 
 template <int R, bool GRAD, bool NARROW>
 __global__ void __launch_bounds__(kRegBlock, depth2_blocks(GRAD, R)) depth2_kernel(const RegLaunch L) {
+    wait_before();
     using CT = Counts<NARROW>;
     constexpr int NP = 1 << (R - 1), NG = 1 << (R - 2), HG = NG / 2, kWarps = kRegBlock / 32;
     constexpr int NOUT = reg_outputs(2, GRAD), G = reg_group(2, GRAD);

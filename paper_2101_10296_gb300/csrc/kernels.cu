@@ -56,6 +56,7 @@ namespace {
 constexpr int kPrepBlock = 64;
 
 __global__ void __launch_bounds__(kPrepBlock) prep_kernel(const PrepArgs a, int parts, int row_blocks, int mix_blocks) {
+    wait_before();
     const int64_t GP = int64_t(a.G) * a.P;
     const int p2 = 2 * a.p;
     if (int(blockIdx.x) < row_blocks) {
@@ -209,6 +210,20 @@ int smem_per_block(int blocks) {
     return v;
 }
 
+cudaError_t launch_after(const void *fn, int grid, int block, void **args, size_t smem, cudaStream_t s) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(unsigned(grid));
+    c.blockDim = dim3(unsigned(block));
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &attr;
+    c.numAttrs = 1;
+    return cudaLaunchKernelExC(&c, fn, args);
+}
+
 cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s) {
     const int64_t rows = int64_t(a.G) * a.P * a.p;
     // segments per table row while rows x segments fit one block per SM
@@ -220,9 +235,10 @@ cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s) {
     if (a.terms) out = std::max<int64_t>(out, a.n_reps * a.P);
     const int64_t out_blocks = std::min<int64_t>(blocks(out), int64_t(sm_count()) * 8);
     if (row_blocks + mix_blocks + out_blocks > INT32_MAX) return cudaErrorInvalidValue;
-    prep_kernel<<<int(row_blocks + mix_blocks + out_blocks), kPrepBlock, 0, s>>>(a, parts, int(row_blocks),
-                                                                                  int(mix_blocks));
-    return cudaGetLastError();
+    PrepArgs arg = a;
+    int rb = int(row_blocks), mb = int(mix_blocks);
+    void *args[] = {&arg, &parts, &rb, &mb};
+    return launch_after((const void *)prep_kernel, int(row_blocks + mix_blocks + out_blocks), kPrepBlock, args, 0, s);
 }
 
 int reg_energy_grid(bool wide, size_t smem) {
@@ -250,11 +266,11 @@ cudaError_t reg_prepare() {
 
 cudaError_t launch_reg_energy(const RegLaunch &a, bool wide, int grid, cudaStream_t s) {
     const size_t sm = reg_smem_bytes(a.jpt, a.p, a.cmax1, false);
-    if (wide)
-        reg_cone_kernel<kRegBitsEnergy, uint64_t, false, 0><<<grid, kRegBlock, sm, s>>>(a);
-    else
-        reg_cone_kernel<kRegBitsEnergy, uint32_t, false, 0><<<grid, kRegBlock, sm, s>>>(a);
-    return cudaGetLastError();
+    RegLaunch arg = a;
+    void *args[] = {&arg};
+    const void *fn = wide ? (const void *)reg_cone_kernel<kRegBitsEnergy, uint64_t, false, 0>
+                          : (const void *)reg_cone_kernel<kRegBitsEnergy, uint32_t, false, 0>;
+    return launch_after(fn, grid, kRegBlock, args, sm, s);
 }
 
 cudaError_t launch_cut_table(const DevCone *cone, uint8_t *out, int32_t n, int32_t *status, cudaStream_t s) {

@@ -28,21 +28,6 @@ const void *grad_fn_for(int p) {
     }
 }
 
-template <int RG, typename MT, int PC>
-void launch(const RegLaunch &a, int grid, size_t sm, cudaStream_t s) {
-    reg_cone_kernel<RG, MT, true, PC><<<grid, kRegBlock, sm, s>>>(a);
-}
-
-template <int RG, typename MT>
-void launch_for(const RegLaunch &a, int grid, size_t sm, cudaStream_t s) {
-    switch (a.p) {
-        case 1: launch<RG, MT, 1>(a, grid, sm, s); break;
-        case 2: launch<RG, MT, 2>(a, grid, sm, s); break;
-        case 3: launch<RG, MT, 3>(a, grid, sm, s); break;
-        default: launch<RG, MT, 0>(a, grid, sm, s); break;
-    }
-}
-
 }  // namespace
 
 template <int RG>
@@ -64,11 +49,10 @@ int reg_grad_grid_r(bool wide, size_t smem, int p) {
 template <int RG>
 cudaError_t launch_reg_grad_r(const RegLaunch &a, bool wide, int grid, cudaStream_t s) {
     const size_t sm = reg_smem_bytes(a.jpt, a.p, a.cmax1, true);
-    if (wide)
-        launch_for<RG, uint64_t>(a, grid, sm, s);
-    else
-        launch_for<RG, uint32_t>(a, grid, sm, s);
-    return cudaGetLastError();
+    RegLaunch arg = a;
+    void *args[] = {&arg};
+    const void *fn = wide ? grad_fn_for<RG, uint64_t>(a.p) : grad_fn_for<RG, uint32_t>(a.p);
+    return launch_after(fn, grid, kRegBlock, args, sm, s);
 }
 
 }  // namespace qaoa

@@ -210,13 +210,11 @@ extern "C" int qaoa_energy_noalloc(const qaoa_plan *plan, int64_t n_points, cons
                 B.n_items = std::min(wave, items - i0);
                 if (bs.split_e) {
                     e = launch_split_wave(B, false, d->chunk_window, launches, s);
-                    B.chained = 1;
                     continue;
                 }
                 for (const BigPass &ps : bs.fwd) {
                     B.pass = ps;
                     e = launch_big_pass(B, false, s);
-                    B.chained = 1;
                     if (e != cudaSuccess) break;
                 }
             }

@@ -114,6 +114,7 @@ struct P1Row {
 template <bool GRAD, int ROW>
 __global__ void __launch_bounds__(kRegBlock, GRAD ? kP1GradMinBlocks : kP1EnergyMinBlocks)
     reg_p1_kernel(const RegLaunch L) {
+    wait_before();
     using T = P1Row<ROW>;
     extern __shared__ __align__(256) unsigned char s_raw[];
     constexpr int kWarps = kRegBlock / 32, kPairs = kP1Blocks / 2;
@@ -249,8 +250,7 @@ cudaError_t reg_p1_prepare() {
 cudaError_t launch_reg_p1(const RegLaunch &a, bool grad, int grid, cudaStream_t s) {
     RegLaunch arg = a;
     void *args[] = {&arg};
-    return cudaLaunchKernel(p1_fn(grad, a.cmax1), dim3(unsigned(grid)), dim3(kRegBlock), args,
-                            reg_p1_smem_bytes(a.jpt, a.cmax1, grad), s);
+    return launch_after(p1_fn(grad, a.cmax1), grid, kRegBlock, args, reg_p1_smem_bytes(a.jpt, a.cmax1, grad), s);
 }
 
 }  // namespace qaoa

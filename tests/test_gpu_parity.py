@@ -880,6 +880,70 @@ def test_one_plan_on_two_streams_at_once(q):
         assert plan.device_status() == 0
 
 
+@pytest.mark.parametrize("before", ["kernel", "copy", "stream"])
+@pytest.mark.parametrize("graphs,p", [
+    ([I.cycle(12)], 1), ([I.random_regular(60, 3, 2)], 2), ([I.random_regular(16, 3, 4)], 3),
+    ([I.circulant(25, [1, 2])], 4),
+], ids=["p1", "p2", "core", "general"])
+def test_evaluations_wait_for_what_stands_before_them(q, graphs, p, before):
+    """The launches of an evaluation are prepared while the launch before them
+    drains: parameters written just before, by a kernel, a copy or on a stream
+    joined by an event, behind work that takes a while, are the ones used, and an
+    output is complete for the operation after; directly and captured."""
+    plan = q.Plan(graphs, p)
+    plan.upload()
+    ths = [_params(np.stack([I.draw_params(p, 3, 31 + k)])) for k in range(3)]
+    ref = [(*plan.energy_grad(th), plan.energy(th)) for th in ths]  # the adjoint kernels' E rounds otherwise
+    slow = torch.ones(1 << 25, device="cuda")
+    th, src, other = torch.zeros_like(ths[0]), torch.zeros_like(ths[0]), torch.cuda.Stream()
+    host = torch.zeros(ths[0].shape, dtype=torch.float64).pin_memory()
+    out = torch.empty(1, 3, dtype=torch.float64, device="cuda")
+    scale = torch.ones((), dtype=torch.float64, device="cuda")
+
+    def evaluate():
+        for _ in range(8):
+            slow.mul_(1.0)
+        if before == "kernel":
+            torch.mul(src, scale, out=th)
+        elif before == "copy":
+            th.copy_(host, non_blocking=True)
+        else:
+            other.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(other):
+                for _ in range(8):
+                    slow.mul_(1.0)
+                torch.mul(src, scale, out=th)
+            torch.cuda.current_stream().wait_stream(other)
+        e, g = plan.energy_grad(th)
+        plan.energy_noalloc(th, out=out)
+        return e * scale, g * scale, out * scale
+
+    def check(got, k):
+        torch.cuda.synchronize()
+        e, g, o = (x.cpu().numpy() for x in got)
+        e0, g0, o0 = (x.cpu().numpy() for x in ref[k])
+        assert np.allclose(e, e0, rtol=1e-12, atol=0) and np.allclose(o, o0, rtol=1e-12, atol=0)
+        assert np.allclose(g, g0, rtol=1e-9, atol=1e-12)
+
+    def fill(k):
+        src.copy_(ths[k])
+        host.copy_(ths[k])
+        th.zero_()
+        torch.cuda.synchronize()
+
+    for k in range(3):
+        fill(k)
+        check(evaluate(), k)
+    graph, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=s):
+        got = evaluate()
+    for k in range(3):
+        fill(k)
+        graph.replay()
+        check(got, k)
+    assert plan.device_status() == 0
+
+
 def test_cuda_graph_replay_matches_direct_calls(q):
     plan, G = _mixed_plan(q)
     assert plan.info()["n_big"] > 0
