@@ -62,12 +62,12 @@ SIDE_SEEDS = (1, 2, 3, 4)
 
 # DRAM bytes per launch of the dominant kernel (the depth-1 adjoint kernel on
 # this workload) from a one-pass ncu capture of `bench.py --case reg-mix48`
-# (dram__bytes_read.sum + dram__bytes_write.sum: 12,878,592 + 0), with the
+# (dram__bytes_read.sum + dram__bytes_write.sum: 12,864,256 + 0), with the
 # hash of the sources they were taken on; a change to any of them reports
 # null until it is captured again.
-TRAFFIC = {"kernels_sha1": "7f85fecc87ccd76559b4bf100cd0afd576bea2e7", "bytes_per_launch": 12878592,
+TRAFFIC = {"kernels_sha1": "93b6940e547d87642455972a6bc63668a0d394c5", "bytes_per_launch": 12864256,
            "source": "ncu one-pass capture (dram__bytes_read.sum + dram__bytes_write.sum) of "
-                     "`python bench.py --case reg-mix48` (default tuning: 12 points per task, 6 blocks per SM), "
+                     "`python bench.py --case reg-mix48` (default tuning, 6 blocks per SM), "
                      "summarised in profiles/reg_p1_mix48_p1.md"}
 
 
@@ -180,7 +180,8 @@ def kernels_sha1():
     """Hash of the dominant kernel's sources (the depth-1 kernel) and of the
     planner and upload code that decide what it reads (the block records)."""
     h = hashlib.sha1()
-    for f in ("p1_kernel.cu", "reg_common.cuh", "device.cuh", "capi.cu", "plan.cpp", "block_orbits.cpp"):
+    for f in ("p1_kernel.cu", "packed.cuh", "dev_math.cuh", "reg_common.cuh", "device.cuh", "capi.cu", "plan.cpp",
+              "block_orbits.cpp"):
         h.update(open(os.path.join(ROOT, "paper_2101_10296_gb300", "csrc", f), "rb").read())
     return h.hexdigest()
 
@@ -648,7 +649,7 @@ def run_ours(args, rank, world, local_rank):
             "energy_grad_evals_per_s": world * s_evals / (s_ms / 1e3),
             "plain_all_edge_evals_per_s": world * s_evals / (sp_ms / 1e3),
             "n_reps": int(splan.info()["n_reps"]), "tuning": s_tuning,
-            # the general adjoint register kernel's algorithmic FP32 work over the whole step
+            # the depth-2 adjoint kernel's algorithmic FP32 work over the whole step
             # (prep_kernel + that kernel), against the same FP32 peak as the roofline
             "fp32_tflops_alg": s_flops / (s_ms / 1e3) / 1e12}
     # the training driver: Adam on -E from 64 starts per graph, timed after a warm-up step

@@ -378,7 +378,9 @@ int qaoa_device_status(const qaoa_plan *plan, int32_t *status);
  *                    larger values are cut to what fits 12 KB per warp; the
  *                    depth-1 kernel's default is what leaves room for its
  *                    resident blocks: the multiprocessor's shared memory
- *                    split among them, less the per-block reservation)
+ *                    split among them, less the per-block reservation; the
+ *                    depth-2 kernel's gives the busiest multiprocessor the
+ *                    least work)
  *   blocks_per_sm    resident blocks per SM of the persistent grid (default:
  *                    the occupancy limit)
  *   big_scratch_bytes scratch per call for large-state cones, which sets how

@@ -97,6 +97,9 @@ __device__ __forceinline__ int popc_w(uint64_t x) { return __popcll(x); }
 // edge that joins them, whatever base is: so a lane counts G + 1 words and adds up
 // the others (two integer additions per value instead of a 64-bit exclusive or, two
 // popcounts and an addition).  The pairs are uniform: pairs[q (q - 1) / 2 + q'].
+// With rounds that leave the swizzle's address work out where there is none: 6x6
+// torus, p = 3, 32 points, energy 8.27 -> 7.49 ms, gradient, 8 points 8.84 -> 8.58
+// (64-bit words); no change with 32-bit words (cubic n = 24).
 constexpr int kPairs5 = 10;
 template <typename MT>
 __device__ __forceinline__ int window_pair(MT a, MT b, MT neg) {

@@ -185,11 +185,12 @@ inline size_t core_smem_bytes(int p, bool grad) { return size_t(4) * (p * kCoreR
 // per tile.  The derivative sums gather per lane in compensated pairs in shared
 // memory meanwhile.
 //
-// Bound: instruction fetch and latency (ncu, adjoint, p = 3: 49% of the issue
-// slots, FP32 pipe 52%, no-instruction the first stall; 5,000 instructions of
-// straight-line code, so that the block's warps start each tile together, which
-// lets them share fetched code: 14.4 -> 13.9 ms; further barriers within the tile or
-// larger blocks were slower), the energy by shuffles and shared memory (55%).  Measured
+// Bound: the adjoint by the operand reads of its packed FMAs (ncu, p = 3: FP32 pipe
+// 63% of the cycles, where packed FMAs of three fresh register pairs reach about 70%,
+// 55% of the issue slots; 5,000 instructions of straight-line code, so that the
+// block's warps start each tile together, which lets them share fetched code: 14.4 ->
+// 13.7 ms; further barriers within the tile or larger blocks were slower), the energy
+// by shuffles and shared memory (61%).  Measured
 // against the unpacked kernel with one tile per task: four cubic graphs n = 24,
 // p = 3, 25 points, gradient 21.6 -> 15.8 ms; 6x6 torus, p = 3, 32 points, energy
 // 10.1 -> 8.8 ms (both with their outer passes).

@@ -385,8 +385,8 @@ int ensure_uploaded(const qaoa_plan *plan) {
 // Register qubits per thread of the adjoint kernel: the tuned value, else by
 // the amount of work.  Five register qubits halve the lane exchanges but need
 // 255 registers (2 blocks of 128 threads per SM), so they win on plans that
-// keep the SMs busy for several waves (measured at p = 2: 10% faster on four
-// random cubic graphs of 2000 vertices, 9% on two random 4-regular ones) and
+// keep the SMs busy for several waves (measured at p = 2: 2.34 against 2.68 ms on
+// four random cubic graphs of 2000 vertices, 9% on two random 4-regular ones) and
 // lose on small ones (11-28% slower on the 8x8 and 100x100 tori, one to three
 // cones).  The untuned choice takes 5 when the 5-qubit work list, at up to 32
 // points per warp task, gives at least four waves of 8 warps per SM.
