@@ -61,8 +61,14 @@ __global__ void __launch_bounds__(kPrepBlock) prep_kernel(const PrepArgs a, int 
     const int p2 = 2 * a.p;
     if (int(blockIdx.x) < row_blocks) {
         // exp(-i gamma c) of one (graph, point, layer), c in the thread's segment: the segment's first
-        // entry directly, then the recurrence z_(c+1) = z_c exp(-i gamma) in FP64 (after at most 64
-        // steps its rounding error, ~1e-14, is far below the FP32 table's own)
+        // entry, then the recurrence z_(c+1) = z_c exp(-i gamma) in FP64 (after at most 64 steps its
+        // rounding error, ~1e-14, is far below the FP32 table's own).  The first entry is not sincos of
+        // the rounded product gamma c0 (off by |gamma c0| 2^-53, more than the table's own rounding from
+        // |gamma| = 1e7 on): up to 2^20 the product's error is put back, beyond it exp(-i gamma), whose
+        // argument sincos reduces exactly, is raised to the power by squarings.  (Squarings throughout
+        // wait for the first sincos instead of running beside it: 11.7 against 10.4 us a replayed
+        // evaluation of the 8x8 torus, p = 2, 8 points; 72.5 against 71.7 for Erdos-Renyi n = 10,000,
+        // p = 1, 101 points, gradient.)
         const int64_t t = int64_t(blockIdx.x) * kPrepBlock + threadIdx.x;
         const int64_t r = t / parts;
         if (r >= GP * a.p) return;
@@ -76,8 +82,28 @@ __global__ void __launch_bounds__(kPrepBlock) prep_kernel(const PrepArgs a, int 
         float2 *row = a.lut + r * a.cmax1;
         double zr = 1.0, zi = 0.0;
         if (c0 > 0) {
-            sincos(gamma * double(c0), &zi, &zr);
-            zi = -zi;
+            const double first = gamma * double(c0);
+            if (fabs(gamma) < 0x1p20) {
+                const double e = fma(gamma, double(c0), -first);  // the product's rounding error, below 2^-27
+                double se, ce;
+                sincos(first, &se, &ce);
+                zr = fma(-se, e, ce);
+                zi = -fma(ce, e, se);
+            } else {
+                double br = cs, bi = -sn;
+                for (int k = c0;;) {
+                    if (k & 1) {
+                        const double nr = fma(zr, br, -(zi * bi));
+                        zi = fma(zr, bi, zi * br);
+                        zr = nr;
+                    }
+                    k >>= 1;
+                    if (k == 0) break;
+                    const double nr = fma(br, br, -(bi * bi));
+                    bi = 2.0 * (br * bi);
+                    br = nr;
+                }
+            }
         }
         for (int c = c0; c < c1; ++c) {
             row[c] = make_float2(float(zr), float(zi));

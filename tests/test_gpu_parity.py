@@ -292,6 +292,27 @@ def test_depth1_kernel_edge_cases(q, P):
     assert plan.device_status() == 0
 
 
+@pytest.mark.parametrize("gamma", [1e6 + 1 / 3, 1e12 + 1 / 3, 1e15 / 3])
+@pytest.mark.parametrize("graph,p", [(I.star(11), 1), (I.star(5), 2), (I.petersen(), 3)])
+@pytest.mark.parametrize("P", [1, 4000])
+def test_large_angles(q, graph, p, P, gamma):
+    """exp(-i gamma C) has period 2 pi in gamma (C is an integer), so a large gamma gives what its
+    reduction gives, whether the call has one point or many (the table kernel cuts the rows of small
+    calls in segments).  Reduced as atan2(sin gamma, cos gamma), to 2^-52 of pi."""
+    n, edges = graph
+    th = I.draw_params(p, P, 17)
+    th[0, 0] = gamma
+    plan = q.Plan(graph, p, orbits=False)
+    e, g = plan.energy_grad(_params(th))
+    red = th[0].copy()
+    red[0] = math.atan2(math.sin(gamma), math.cos(gamma))
+    eref, gref = O.orbit_grad_adjoint(n, edges, red, p, np.arange(len(edges)))
+    assert abs(e[0, 0].item() - eref) <= E_REL_TOL * abs(eref)
+    assert abs(plan.energy(_params(th))[0, 0].item() - eref) <= E_REL_TOL * abs(eref)
+    _check_grad(g[0, 0].cpu().numpy(), gref, energy=eref)
+    assert plan.device_status() == 0
+
+
 @pytest.mark.parametrize("graph,p,kw", [
     (I.random_regular(30, 3, 1), 1, {}),                     # depth-1 kernel
     (I.petersen(), 2, {}),                                   # general register kernel
