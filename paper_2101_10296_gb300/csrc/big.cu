@@ -24,8 +24,8 @@ constexpr int NW = 8;                       // packed cut counts, 4 registers pe
 // shared memory, a lane holds the cut word of one address bit outside the window
 // (a tile's fixed word is one XOR reduction), cut values are counted once per
 // tile (bytes of kCoreScale c), and the derivative sums gather per lane in
-// compensated pairs in shared memory until the item's tiles are done.  Sums over
-// the registers run in register order: lower halves, then upper ones.
+// shared memory (Tfl) until the item's tiles are done.  Sums over the registers run
+// in register order: lower halves, then upper ones.
 //
 // Bound: FP32 and latency at two blocks per SM (three, with 168 registers, spill:
 // 1.96 against 1.24 ms).  Against scalar registers, a popcount per amplitude and
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(128) big_pass_kernel(const __grid_constant__ B
     const int64_t block_amps = int64_t(1) << nin;
     const int64_t lowmask = (int64_t(1) << (b - 5)) - 1;
     unsigned char *tab = s_big + warp * (p * kCoreRow);
-    float2 *sums = reinterpret_cast<float2 *>(s_big + 4 * (p * kCoreRow)) + warp * (2 * p * 32) + lane;
+    float *sums = reinterpret_cast<float *>(s_big + 4 * (p * kCoreRow)) + warp * (2 * p * kTileSum) + lane;
     const uint32_t tab0 = smem_addr(tab);
     for (int64_t task = gw; task < ntask; task += nw) {
         const int64_t it = task / per_item;
@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(128) big_pass_kernel(const __grid_constant__ B
         __syncwarp();
         stage_rows(tab, L.lut + gj * p * L.cmax1, p, L.cmax1, lane);
         if (GRAD)
-            for (int c = 0; c < 2 * p; ++c) sums[32 * c] = make_float2(0.f, 0.f);
+            for (int c = 0; c < 2 * p; ++c) tile_sum_clear(sums + kTileSum * c);
         __syncwarp();
         // cut words: shell block ^ lane part, the address bits outside the window (one per lane), the window's
         float mult = 1.f;
@@ -82,13 +82,8 @@ __global__ void __launch_bounds__(128) big_pass_kernel(const __grid_constant__ B
         const float sig = __int_as_float((127 - C->n) << 23);  // 2^-n
         // Im<r|x> = 0: C - m/2 in place of C in the derivatives
         const float b0 = 8388608.f + 0.5f * kCoreScale * float(C->m);
-        auto add_sum = [&](int c, Dfl v) {
-            const float2 s = sums[32 * c];
-            Dfl a{s.x, s.y};
-            dfl_add(a, v);
-            sums[32 * c] = make_float2(a.hi, a.lo);
-        };
-        Dfl e_sum{0.f, 0.f}, t_sum{0.f, 0.f};
+        auto add_sum = [&](int c, Dfl v) { tile_sum_add(sums + kTileSum * c, v); };
+        double e_sum = 0.0, t_sum = 0.0;  // of the warp's tile sums
         for (int64_t tile = tile0; tile < tile0 + tpw; ++tile) {
             // inner index of (lane, register i): xb | (i << b) | lane
             const int64_t xb = ((tile & lowmask) << 5) | ((tile >> (b - 5)) << (b + 5));
@@ -156,8 +151,8 @@ __global__ void __launch_bounds__(128) big_pass_kernel(const __grid_constant__ B
 #pragma unroll
                         for (int h = 0; h < NP; ++h) acc = fmaf(hi(x[h].r), hi(x[h].r), fmaf(hi(x[h].i), hi(x[h].i), acc));
                         const float tv = sg * acc * sig * mult;  // this block's share of <Z_0 Z_1>
-                        dfl_add(e_sum, warp_sum(-0.5f * float(C->weight) * tv));
-                        if (L.terms) dfl_add(t_sum, warp_sum(tv));
+                        e_sum += f2d(warp_sum(-0.5f * float(C->weight) * tv));
+                        if (L.terms) t_sum += f2d(warp_sum(tv));
                         break;
                     }
                     case kOpLamInit: {
@@ -247,14 +242,13 @@ __global__ void __launch_bounds__(128) big_pass_kernel(const __grid_constant__ B
             if (GRAD && (op.type == kOpUnmix || op.type == kOpUnphase)) {
                 // an op's sums, once: a layer's mixer may come in several ops of a pass
                 const int c = op.type == kOpUnmix ? p + op.layer : op.layer;
-                const float2 s = sums[32 * c];
-                sums[32 * c] = make_float2(0.f, 0.f);
-                add_gp(Dfl{s.x, s.y}, 2.f * wgt * sig, L.grad, gj * 2 * p + c);
+                add_gp(tile_sum(sums + kTileSum * c), 2.f * wgt * sig, L.grad, gj * 2 * p + c);
+                tile_sum_clear(sums + kTileSum * c);
             }
         }
         if (reduces && lane == 0) {
-            atomicAdd(L.energy + gj, dfl_value(e_sum));
-            if (L.terms) atomicAdd(L.terms + C->rep * L.P + j, dfl_value(t_sum));
+            atomicAdd(L.energy + gj, e_sum);
+            if (L.terms) atomicAdd(L.terms + C->rep * L.P + j, t_sum);
         }
     }
 }
@@ -343,7 +337,7 @@ cudaError_t launch_big_pass(BigLaunch a, bool grad, cudaStream_t s) {
         void *args[] = {&a};
         return launch_after((const void *)big_mix_kernel, int(std::min<int64_t>(mix_grid(), need)), 128, args, 0, s);
     }
-    const size_t smem = size_t(4) * (a.p * kCoreRow + (grad ? 2 * a.p * 32 * sizeof(float2) : 0));
+    const size_t smem = size_t(4) * (a.p * kCoreRow + (grad ? 2 * a.p * kTileSum * sizeof(float) : 0));
     const void *fn = pass_fn(grad, a.cmax1 - 1 > 32);
     const int full = occupancy_grid(fn, 128, smem);
     a.tpw = tiles_per_task(a.n_items, bits, full);

@@ -195,6 +195,19 @@ __device__ __forceinline__ void add_gp(Dfl v, float w, double *base, int64_t idx
     if ((threadIdx.x & 31) == 0) atomicAdd(base + idx, dfl_value(v));
 }
 
+// Derivative sums of a warp's tiles in shared memory: per output and lane a Tfl, its
+// parts 32 floats apart (s points at the lane's first).
+constexpr int kTileSum = 96;
+__device__ __forceinline__ void tile_sum_clear(float *s) { s[0] = s[32] = s[64] = 0.f; }
+__device__ __forceinline__ void tile_sum_add(float *s, Dfl v) {
+    Tfl a{s[0], s[32], s[64]};
+    tfl_add(a, v);
+    s[0] = a.hi;
+    s[32] = a.lo;
+    s[64] = a.lo2;
+}
+__device__ __forceinline__ Dfl tile_sum(const float *s) { return tfl_pair(Tfl{s[0], s[32], s[64]}); }
+
 // Item -> (cone of the shape, point j, shell block y).  Cone c owns the items
 // P * [ystart[c], ystart[c+1]), ordered point-major.
 __device__ __forceinline__ void decode_item(const BigLaunch &L, int64_t item, int &ci, int64_t &j, int64_t &y) {

@@ -177,13 +177,13 @@ __host__ __device__ constexpr float zz_sign(int i) { return ((i ^ (i >> 1)) & 1)
 // ms on the 6x6 torus).
 constexpr int kCoreGradBlocks = 3, kCoreEnergyBlocks = 4;
 
-inline size_t core_smem_bytes(int p, bool grad) { return size_t(4) * (p * kCoreRow + (grad ? 2 * p * 32 * sizeof(float2) : 0)); }
+inline size_t core_smem_bytes(int p, bool grad) { return size_t(4) * (p * kCoreRow + (grad ? 2 * p * kTileSum * sizeof(float) : 0)); }
 
 // A warp takes L.tpw consecutive tiles of one item: the item's decoding, its
 // phase tables (staged in shared memory, rows of real parts and of imaginary
 // parts) and the warp reductions and atomics of the sums are per item and not
-// per tile.  The derivative sums gather per lane in compensated pairs in shared
-// memory meanwhile.
+// per tile.  Meanwhile the tiles' energies and terms gather in FP64, their derivatives
+// per lane in shared memory (Tfl).
 //
 // Bound: the adjoint by the operand reads of its packed FMAs (ncu, p = 3: FP32 pipe
 // 63% of the cycles, where packed FMAs of three fresh register pairs reach about 70%,
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
     const int64_t ntask = L.n_items * per_item;
     const int64_t block_amps = int64_t(1) << nin;
     unsigned char *tab = s_core + warp * (p * kCoreRow);
-    float2 *sums = reinterpret_cast<float2 *>(s_core + (blockDim.x >> 5) * (p * kCoreRow)) + warp * (2 * p * 32) + lane;
+    float *sums = reinterpret_cast<float *>(s_core + (blockDim.x >> 5) * (p * kCoreRow)) + warp * (2 * p * kTileSum) + lane;
     const uint32_t tab0 = smem_addr(tab);
     // the block's warps start every tile together (a warp past the last task, or of a
     // foreign shape, only keeps step)
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
         {
             stage_rows(tab, L.lut + gj * p * L.cmax1, p, L.cmax1, lane);
             if (GRAD)
-                for (int c = 0; c < 2 * p; ++c) sums[32 * c] = make_float2(0.f, 0.f);
+                for (int c = 0; c < 2 * p; ++c) tile_sum_clear(sums + kTileSum * c);
         }
         __syncwarp();
         // cut word of the item's fixed bits: shell block, lane qubits
@@ -248,13 +248,8 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
         // (the mean cut value) removes most of the cancellation in the FP32
         // sums.  Counts are bytes of kCoreScale c; 2^23 + kCoreScale c0 here.
         const float b0 = 8388608.f + 0.5f * kCoreScale * float(C->m);
-        auto add_sum = [&](int c, Dfl v) {
-            const float2 s = sums[32 * c];
-            Dfl a{s.x, s.y};
-            dfl_add(a, v);
-            sums[32 * c] = make_float2(a.hi, a.lo);
-        };
-        Dfl e_sum{0.f, 0.f}, t_sum{0.f, 0.f};  // of the warp's tile sums
+        auto add_sum = [&](int c, Dfl v) { tile_sum_add(sums + kTileSum * c, v); };
+        double e_sum = 0.0, t_sum = 0.0;  // of the warp's tile sums
         for (int64_t u = u0; u < u0 + tpw; ++u) {
             __syncthreads();
             if (!ours) continue;
@@ -324,8 +319,8 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
             }
             {
                 const float tv = acc * sig * mult;  // this tile's share of <Z_0 Z_1>
-                dfl_add(e_sum, warp_sum(-0.5f * wgt * tv));
-                if (L.terms) dfl_add(t_sum, warp_sum(tv));
+                e_sum += f2d(warp_sum(-0.5f * wgt * tv));
+                if (L.terms) t_sum += f2d(warp_sum(tv));
             }
             if (GRAD) {
                 C2 r[NP];
@@ -404,16 +399,16 @@ __global__ void __launch_bounds__(128, GRAD ? kCoreGradBlocks : kCoreEnergyBlock
         }
         if (!ours) continue;
         if (lane == 0) {
-            atomicAdd(L.energy + gj, dfl_value(e_sum));
-            if (L.terms) atomicAdd(L.terms + C->rep * L.P + j, dfl_value(t_sum));
+            atomicAdd(L.energy + gj, e_sum);
+            if (L.terms) atomicAdd(L.terms + C->rep * L.P + j, t_sum);
         }
         if (GRAD) {
             const float wgt2 = 2.f * wgt * mult * sig0;
             for (int l = 1; l < p; ++l) {
-                add_gp(Dfl{sums[32 * (p + l)].x, sums[32 * (p + l)].y}, wgt2, L.grad, gj * 2 * p + p + l);
-                add_gp(Dfl{sums[32 * l].x, sums[32 * l].y}, wgt2, L.grad, gj * 2 * p + l);
+                add_gp(tile_sum(sums + kTileSum * (p + l)), wgt2, L.grad, gj * 2 * p + p + l);
+                add_gp(tile_sum(sums + kTileSum * l), wgt2, L.grad, gj * 2 * p + l);
             }
-            add_gp(Dfl{sums[32 * p].x, sums[32 * p].y}, wgt2, L.grad, gj * 2 * p + p);
+            add_gp(tile_sum(sums + kTileSum * p), wgt2, L.grad, gj * 2 * p + p);
         }
     }
 }
@@ -432,7 +427,7 @@ __device__ __forceinline__ int qubit_of(int a, int rb) { return a < 5 ? rb + a :
 // registers = the window).  The item's first-layer table sits in shared memory,
 // a lane holds the cut word of one address bit outside the window (a tile's
 // fixed word is one XOR reduction), and the derivative sums gather over the
-// tiles.  The state is held an amplitude per packed pair; kOuterFirst, which
+// tiles (Tfl).  The state is held an amplitude per packed pair; kOuterFirst, which
 // forms pair terms, holds registers h and h + 16 together as the core pass does.
 // Blocks per SM: 4 and 3 (generation at 3 and 5, the others at 2 and 4: no faster).
 // Generation was bound by the integer pipe (64-bit popcounts and table lookups in
@@ -497,7 +492,7 @@ __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_ke
 #pragma unroll
                 for (int t = 0; t < q; ++t) pairs[q * (q - 1) / 2 + t] = uniform(window_pair(col[q], col[t], MT(C->neg)));
         }
-        Dfl s_dg{0.f, 0.f}, s_db{0.f, 0.f};
+        Tfl s_dg{0.f, 0.f, 0.f}, s_db{0.f, 0.f, 0.f};  // of the lane's tiles
         for (int64_t tile = tile0; tile < tile0 + tpw; ++tile) {
             // address of (lane, register i) = xb | (i << b) | lane
             const int64_t xb = ((tile & lowmask) << 5) | ((tile >> (b - 5)) << (b + 5));
@@ -541,7 +536,7 @@ __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_ke
                 }
 #pragma unroll
                 for (int h = 0; h < 16; ++h) dg = fmaf(uw[h], uv[h], dg);
-                dfl_add(s_dg, Dfl{dg, 0.f});
+                tfl_add(s_dg, Dfl{dg, 0.f});
                 if (outer_terms) {
                     Dfl db{0.f, 0.f};
 #pragma unroll
@@ -574,7 +569,7 @@ __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_ke
                         for (int h = 0; h < 16; ++h) t += uv[h];
                         dfl_add(db, t);
                     }
-                    dfl_add(s_db, db);
+                    tfl_add(s_db, db);
                 }
             } else {
                 P2 x[32];
@@ -600,8 +595,8 @@ __global__ void __launch_bounds__(128, MODE == kOuterGen ? 4 : 3) split_outer_ke
         if (MODE == kOuterFirst) {
             // lambda = 2^(-n/2) kappa_1^(2 n_in) x once the first mixer is undone
             const float wgt2 = 2.f * float(C->weight) * mult * __int_as_float((127 - C->n) << 23) * f1.k2n;
-            add_gp(s_dg, wgt2, L.grad, gj * 2 * p);
-            if (p > 1) add_gp(s_db, wgt2, L.grad, gj * 2 * p + p);
+            add_gp(tfl_pair(s_dg), wgt2, L.grad, gj * 2 * p);
+            if (p > 1) add_gp(tfl_pair(s_db), wgt2, L.grad, gj * 2 * p + p);
         }
     }
 }

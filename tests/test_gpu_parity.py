@@ -656,6 +656,27 @@ def test_chunk_passes_in_many_waves_and_cuda_graph(q):
     assert plan.device_status() == 0 and fresh.device_status() == 0
 
 
+@pytest.mark.parametrize("kw", [{}, {"big_general": True}], ids=["core-tile", "general"])
+def test_tiles_gather_without_loss(q, kw):
+    """How many tiles of a block a warp takes before it adds to the outputs (up to 64 of K_{8,8}'s 64 or
+    128 in a large wave, one in waves of 28 MiB) does not show in the results: the tiles' sums gather
+    with FP64's bits.  A point's 128 additions, grouped one way and the other, differ by sqrt(256 / 12) 2^-53 of the
+    sum at most (rms, independent roundings), and the pairs in which the lanes meet by 2^-48 of a tile's
+    sum each: 2^-48 of the components' rms bounds both.  FP32 pairs over the tiles gave 2^-46."""
+    n, edges = I.complete_bipartite(8, 8)
+    plan = q.Plan((n, edges), 2, **kw)
+    th = _params(I.draw_params(2, 2048, 3))
+    out = []
+    for budget in (28 << 20, 1 << 30):
+        plan.set_tuning(big_scratch_bytes=budget)
+        e, g, t = plan.energy_grad(th, terms=True)
+        e2, t2 = plan.energy(th, terms=True)
+        out.append([x.cpu().numpy().reshape(2048, -1) for x in (e, g[0], t, e2, t2)])
+    for a, b in zip(*out):
+        assert np.all(np.sqrt(((a - b) ** 2).mean(0)) <= 2.0 ** -48 * np.sqrt((a ** 2).mean(0)))
+    assert plan.device_status() == 0
+
+
 @pytest.mark.parametrize("graphs,p", [([I.random_regular(200, 3, s) for s in (1, 2)], 2),
                                       ([I.erdos_renyi(150, 4 / 149, 3), I.circulant(40, [1, 3])], 1),
                                       ([I.random_regular(24, 3, s) for s in (1, 2)], 3)])
