@@ -53,9 +53,9 @@ cudaError_t build_depth2_records(const DevCone *cones, const uint64_t *shell, co
                                  const int64_t *start, int64_t slots, int R, int cmax1, uint32_t *cnt, float *wk) {
     const int64_t n = slots << (R - 2);
     const int64_t blocks = std::min<int64_t>((n + 255) / 256, 65535);
-    depth2_records_kernel<<<int(blocks), 256>>>(cones, shell, slot_cone, start, slots, R,
-                                                 depth2_narrow(cmax1) ? 4 : 2, cnt, wk);
-    return cudaGetLastError();
+    int scale = depth2_narrow(cmax1) ? 4 : 2;
+    void *args[] = {&cones, &shell, &slot_cone, &start, &slots, &R, &scale, &cnt, &wk};
+    return launch((const void *)depth2_records_kernel, int(blocks), 256, args, nullptr);
 }
 
 template cudaError_t depth2_prepare_r<kRegBitsEnergy, false>();

@@ -154,6 +154,10 @@ struct PrepArgs {
 // 115; n = 20, 4 points, gradient 375 -> 348; circulant n = 30, p = 4, 64 points,
 // gradient 1233 -> 1217.
 cudaError_t launch_after(const void *fn, int grid, int block, void **args, size_t smem, cudaStream_t s);
+// A plain launch.  Both answer for the launch itself: cudaGetLastError() would also
+// give an error that an earlier call met and reported (scratch refused by the
+// allocator, say).
+cudaError_t launch(const void *fn, int grid, int block, void **args, cudaStream_t s);
 cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s);
 // wide = some cone has more than 32 edges (64-bit cut words).  Dynamic
 // shared memory: 4 warps x jpt x p x cmax1 float2 (phase tables).

@@ -250,6 +250,10 @@ cudaError_t launch_after(const void *fn, int grid, int block, void **args, size_
     return cudaLaunchKernelExC(&c, fn, args);
 }
 
+cudaError_t launch(const void *fn, int grid, int block, void **args, cudaStream_t s) {
+    return cudaLaunchKernel(fn, dim3(unsigned(grid)), dim3(unsigned(block)), args, 0, s);
+}
+
 cudaError_t launch_prep(const PrepArgs &a, cudaStream_t s) {
     const int64_t rows = int64_t(a.G) * a.P * a.p;
     // segments per table row while rows x segments fit one block per SM
@@ -303,8 +307,8 @@ cudaError_t launch_cut_table(const DevCone *cone, uint8_t *out, int32_t n, int32
     int64_t threads = int64_t(1) << (n > kRegBitsEnergy ? n - kRegBitsEnergy : 0);
     int64_t blocks = (threads + 127) / 128;
     if (blocks > 65535) blocks = 65535;
-    cut_table_kernel<uint64_t><<<int(blocks), 128, 0, s>>>(cone, out, n, status);
-    return cudaGetLastError();
+    void *args[] = {&cone, &out, &n, &status};
+    return launch((const void *)cut_table_kernel<uint64_t>, int(blocks), 128, args, s);
 }
 
 }  // namespace qaoa

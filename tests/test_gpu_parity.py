@@ -1387,6 +1387,40 @@ def test_injected_allocation_failure_is_reported_and_recoverable(q):
     assert np.allclose(e1.cpu().numpy(), e0, rtol=E_REL_TOL, atol=0) and plan.device_status() == 0
 
 
+@pytest.mark.parametrize("call", ["upload", "cut_table", "energy"])
+def test_scratch_that_does_not_exist_fails_its_own_call_alone(q, call):
+    """A large-state call whose scratch is more than the device has (asked for by big_scratch_bytes) is
+    refused by the allocator and returns QAOA_E_OOM; the next call of any kind answers for itself."""
+    graph = I.petersen()
+    other = q.Plan(graph, 2, orbits=False)
+    theta = I.draw_params(2, 3, 0)
+    if call != "upload":
+        other.upload()
+    big = q.Plan(I.torus(6, 6), 3)
+    P = 1 << 14
+    th = _params(I.draw_params(3, P, 1))
+    big.upload()
+    need = int(big.shell_blocks().sum()) * P * 8 << 18
+    assert need > 4 * torch.cuda.get_device_properties(0).total_memory
+    big.set_tuning(big_scratch_bytes=need)
+    with pytest.raises(q.QAOAError) as ei:
+        big.energy(th)
+    assert ei.value.code == q.QAOA_E_OOM
+    if call == "upload":
+        other.upload()
+    if call == "cut_table":
+        table = other.cut_table(0).cpu().numpy()
+        assert table[0] == 0 and table.max() > 0
+    e = other.energy(_params(theta)).cpu().numpy()[0]
+    for j in range(3):
+        eref = O.lightcone_energy(*graph, theta[j], 2)
+        assert abs(e[j] - eref) <= E_REL_TOL * eref
+    big.set_tuning()
+    e3 = big.energy(th[:, :2]).cpu().numpy()[0]
+    assert np.all(np.abs(e3 - q.Plan(I.torus(6, 6), 3).energy(th[:, :2]).cpu().numpy()[0]) <= E_REL_TOL * 36)
+    assert big.device_status() == 0 and other.device_status() == 0
+
+
 # ------------------------------------- gradients where they are hardest
 
 def _golden(name):
