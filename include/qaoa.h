@@ -26,7 +26,9 @@
  *     NULL = legacy default stream) and is asynchronous: outputs are ready
  *     when the stream reaches that point.
  *   - A plan is immutable after qaoa_plan_upload and may be used from
- *     several streams at once; each call gets its own stream-ordered scratch.
+ *     several streams at once; each call gets its own stream-ordered scratch,
+ *     from a memory pool of the library's own that keeps a bounded amount of
+ *     freed memory between calls (qaoa_plan_set_scratch_keep).
  */
 #ifndef QAOA_H
 #define QAOA_H
@@ -278,6 +280,23 @@ int qaoa_edge_orbits(int32_t n_vertices, int64_t n_edges, const int32_t *edges,
 int qaoa_plan_upload(qaoa_plan *plan);
 
 /*
+ * Device memory that may stay with the library between calls.  The scratch of
+ * a plan's calls comes from one memory pool per device; when a call's scratch
+ * is freed the pool keeps up to the largest `bytes` of the device's uploaded
+ * plans (QAOA_SCRATCH_KEEP_MB for a plan that has set none), outside any other
+ * allocator's accounting, and gives back the rest at the next synchronisation
+ * and all of it when the last plan is freed.  A call waits 0.2 ms (2.5 ms with
+ * large-state scratch) for memory that was not kept.
+ *   bytes  0: none.  The plan's scratch then comes from the device's current
+ *          memory pool (cudaDeviceSetMemPool, else its default pool, which
+ *          gives freed memory back at every synchronisation).
+ * Uploads the plan if needed; not to be called while a call of the plan is
+ * being made.  Errors: QAOA_E_INVALID for bytes < 0, and as qaoa_plan_upload.
+ */
+#define QAOA_SCRATCH_KEEP_MB 2048
+int qaoa_plan_set_scratch_keep(qaoa_plan *plan, int64_t bytes);
+
+/*
  * Integer cut table of one representative's cone (Sec. 2.4: the MaxCut
  * Hamiltonian is diagonal with value C(z) = number of cone edges (a, b) with
  * z_a != z_b; bit q of z is local qubit q).  out_dev: device uint8[2^n]
@@ -385,7 +404,9 @@ int qaoa_device_status(const qaoa_plan *plan, int32_t *status);
  *                    the occupancy limit)
  *   big_scratch_bytes scratch per call for large-state cones, which sets how
  *                    many state blocks a wave holds (default 1 GiB; a wave
- *                    that fits the 129 MB L2 keeps its passes on chip)
+ *                    that fits the 129 MB L2 keeps its passes on chip; what
+ *                    stays allocated between calls is bounded apart from it,
+ *                    by qaoa_plan_set_scratch_keep)
  *   reg_bits_grad    register qubits per thread of the adjoint register
  *                    kernel, 4 or 5: a tile of 2^(bits + 5) amplitudes per
  *                    warp, 5 holding twice the amplitudes per thread at half

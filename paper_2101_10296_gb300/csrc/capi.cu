@@ -6,6 +6,7 @@
 #include <cstring>
 #include <mutex>
 #include <numeric>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -30,25 +31,27 @@ int cuda_fail(cudaError_t e, const char *what) {
 // Stream-ordered scratch of the calls comes from a memory pool of the library's
 // own, one per device.  A pool with release threshold 0 (the device's default
 // pool) gives all its memory back at every synchronisation, and mapping it again
-// cost the next call 0.2 ms (2.5 ms with large-state scratch); this one keeps up
-// to kPoolKeep bytes while the device holds an uploaded plan and gives them back
-// with the last.
-constexpr uint64_t kPoolKeep = uint64_t(2) << 30;
+// cost the next call 0.2 ms (2.5 ms with large-state scratch); this one keeps as
+// much as any of the device's uploaded plans asks for (qaoa_plan_set_scratch_keep)
+// and gives it back with the last.
 constexpr int kPoolDevices = 64;
 struct DevicePool {
     cudaMemPool_t pool = nullptr;
-    int64_t plans = 0;
+    std::multiset<uint64_t> keep;  // of the plans that use it
 };
 std::mutex g_pool_mu;
 DevicePool g_pools[kPoolDevices];
 
-void pool_keep(cudaMemPool_t pool, uint64_t bytes) {
-    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &bytes);
+// Lets the pool hold what its plans ask for; called with g_pool_mu held.
+void pool_hold(DevicePool &d) {
+    uint64_t bytes = d.keep.empty() ? 0 : *d.keep.rbegin();
+    cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &bytes);
+    cudaMemPoolTrimTo(d.pool, bytes);  // what is still in flight goes at the next synchronisation
 }
 
-// The device's pool for one more uploaded plan; null (the default pool serves) if
-// it cannot be made.
-cudaMemPool_t pool_retain(int dev) {
+// The device's pool for one more plan, keeping `bytes`; null (the device's current
+// pool serves) if it cannot be made.
+cudaMemPool_t pool_retain(int dev, uint64_t bytes) {
     if (dev < 0 || dev >= kPoolDevices) return nullptr;
     std::lock_guard<std::mutex> lk(g_pool_mu);
     DevicePool &d = g_pools[dev];
@@ -64,17 +67,16 @@ cudaMemPool_t pool_retain(int dev) {
             return nullptr;
         }
     }
-    if (d.plans++ == 0) pool_keep(d.pool, kPoolKeep);
+    d.keep.insert(bytes);
+    pool_hold(d);
     return d.pool;
 }
 
-void pool_release(int dev) {
+void pool_release(int dev, uint64_t bytes) {
     std::lock_guard<std::mutex> lk(g_pool_mu);
     DevicePool &d = g_pools[dev];
-    if (--d.plans == 0) {
-        pool_keep(d.pool, 0);  // what is still in flight goes at the next synchronisation
-        cudaMemPoolTrimTo(d.pool, 0);
-    }
+    d.keep.erase(d.keep.find(bytes));
+    pool_hold(d);
 }
 
 cudaError_t scratch_alloc(const qaoa_device_plan *d, void **ptr, size_t bytes, cudaStream_t s) {
@@ -694,7 +696,7 @@ extern "C" void qaoa_device_release(qaoa_plan *plan) {
         cudaEventDestroy(pr.second);
     }
     if (cur >= 0) cudaSetDevice(cur);
-    if (d->pool) pool_release(d->device);
+    if (d->pool) pool_release(d->device, d->keep);
     delete d;
     plan->dev = nullptr;
 }
@@ -810,7 +812,7 @@ extern "C" int qaoa_plan_upload(qaoa_plan *plan) {
         shape->ystart.push_back(shape->ystart.back() + c.n_blocks);
     }
     cudaGetDevice(&d->device);
-    d->pool = pool_retain(d->device);
+    d->pool = pool_retain(d->device, d->keep);
     d->n_cones = int64_t(hc.size());
     d->cmax1 = cmax + 1;
     for (const Cone &c : plan->cones) d->n_kpow = std::max(d->n_kpow, c.n_in + 1);
@@ -1041,6 +1043,22 @@ extern "C" int qaoa_plan_set_tuning(qaoa_plan *plan, const qaoa_tuning_t *t) {
     plan->dev->big_budget = t->big_scratch_bytes > 0 ? size_t(t->big_scratch_bytes) : size_t(1) << 30;
     plan->dev->reg_bits_grad = t->reg_bits_grad;
     plan->dev->chunk_window = t->chunk_window > 0 ? t->chunk_window : 10;
+    return QAOA_OK;
+}
+
+extern "C" int qaoa_plan_set_scratch_keep(qaoa_plan *plan, int64_t bytes) {
+    if (!plan || bytes < 0) {
+        set_error("need a plan and bytes >= 0");
+        return QAOA_E_INVALID;
+    }
+    int rc = ensure_uploaded(plan);
+    if (rc != QAOA_OK) return rc;
+    qaoa_device_plan *d = plan->dev;
+    cudaMemPool_t old = d->pool;
+    const uint64_t was = d->keep;
+    d->keep = uint64_t(bytes);
+    d->pool = bytes > 0 ? pool_retain(d->device, d->keep) : nullptr;
+    if (old) pool_release(d->device, was);
     return QAOA_OK;
 }
 

@@ -34,7 +34,8 @@ struct BigShape {
 
 struct qaoa_device_plan {
     int device = -1;
-    cudaMemPool_t pool = nullptr;  // the device's scratch pool (capi.cu), or null: the default pool
+    cudaMemPool_t pool = nullptr;  // the device's scratch pool (capi.cu), or null: the device's current pool
+    uint64_t keep = uint64_t(QAOA_SCRATCH_KEEP_MB) << 20;  // what the scratch pool may hold for this plan
     qaoa::DevCone *cones = nullptr;
     int64_t n_cones = 0;
     // Work lists with 4 and 5 register qubits per thread: the energy takes 5, the

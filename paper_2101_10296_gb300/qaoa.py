@@ -86,6 +86,7 @@ _SIGS = {
     "qaoa_plan_timing": (C.c_int, [_P, C.c_int32]),
     "qaoa_plan_set_tuning": (C.c_int, [_P, C.POINTER(Tuning)]),
     "qaoa_plan_get_tuning": (C.c_int, [_P, C.POINTER(Tuning)]),
+    "qaoa_plan_set_scratch_keep": (C.c_int, [_P, C.c_int64]),
     "qaoa_graph_create": (C.c_int, [_P, C.c_int64, _P, _P, _P, _P, C.POINTER(_P)]),
     "qaoa_graph_launch": (C.c_int, [_P, _P]),
     "qaoa_graph_free": (None, [_P]),
@@ -398,6 +399,11 @@ class Plan:
         t = Tuning()
         _check(lib().qaoa_plan_get_tuning(self._h, C.byref(t)))
         return {k: getattr(t, k) for k, _ in Tuning._fields_}
+
+    def set_scratch_keep(self, nbytes):
+        """Device memory the library may keep between this plan's calls (0: none, scratch comes
+        from the device's current memory pool); see qaoa_plan_set_scratch_keep."""
+        _check(lib().qaoa_plan_set_scratch_keep(self._h, nbytes))
 
     def graph(self, params, grad=True, terms=False):
         """A captured CUDA graph of one evaluation with fixed buffers (see PlanGraph)."""

@@ -1421,6 +1421,47 @@ def test_scratch_that_does_not_exist_fails_its_own_call_alone(q, call):
     assert big.device_status() == 0 and other.device_status() == 0
 
 
+def test_scratch_kept_between_calls_is_bounded_and_given_back(q):
+    """Device memory that stays allocated after a large-state call (1 GiB of scratch): none where the
+    plan asks for none, at most the default's 2 GiB also after a call with 4 GiB of scratch, and none
+    once the last plan is freed.  32 MiB of slack for what else the process maps."""
+    import gc
+    gc.collect()
+    slack = 32 << 20
+    graph = I.torus(6, 6)
+    th = _params(I.draw_params(3, 24, 2))
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    warm = q.Plan(graph, 3)
+    e0 = warm.energy(th).cpu().numpy()  # loads the kernels
+    warm.close()
+    plan = q.Plan(graph, 3)
+    plan.set_scratch_keep(0)
+    before = free()
+    for keep, scratch, most in ((0, 1 << 30, 0), (None, 1 << 30, 2 << 30), (None, 4 << 30, 2 << 30), (1 << 28, 1 << 30, 1 << 28)):
+        other = plan if keep == 0 else q.Plan(graph, 3)
+        if keep:
+            other.set_scratch_keep(keep)
+        other.set_tuning(big_scratch_bytes=scratch)
+        e = other.energy(th).cpu().numpy()
+        assert np.allclose(e, e0, rtol=E_REL_TOL, atol=0)
+        held = before - free()
+        assert held <= most + slack, (keep, scratch, held)
+        if keep is None:
+            assert held >= 1 << 29, held  # it is kept: the next call does not wait for it
+            other.set_scratch_keep(0)
+            assert before - free() <= slack
+        if other is not plan:
+            other.close()
+        assert before - free() <= slack
+    with pytest.raises(q.QAOAError):
+        plan.set_scratch_keep(-1)
+    assert plan.device_status() == 0
+
+
 # ------------------------------------- gradients where they are hardest
 
 def _golden(name):
