@@ -5,11 +5,12 @@ time (coordinate descent, each group timed with the best values found for
 the groups before it):
 
 1. the number of parameter points a warp task of the register kernels
-   evaluates (1, 2, 4, 8, 12, 16, 32 while the phase tables fit) and the persistent grid's
-   blocks per SM;
-2. with gradients and register-resident cones on the general register
-   kernel (not depth-1 plans): the adjoint register kernel's tile,
-   2^(bits + 5) amplitudes per warp with 4 or 5 register qubits per thread;
+   evaluates (0, the library's own choice for the plan and the number of points,
+   or 1, 2, 4, 8, 12, 16, 32; values past what the kernel's shared memory holds
+   are cut by the library) and the persistent grid's blocks per SM;
+2. with gradients and register-resident cones (not depth-1 plans): the adjoint
+   register kernel's tile, 2^(bits + 5) amplitudes per warp with 4 or 5 register
+   qubits per thread (the depth-2 and the general kernel);
 3. with large-state cones: the scratch per call, i.e. how many state blocks a
    wave holds (waves that fit the L2 keep their passes on chip), and the
    widest window of outer qubits a shared-memory chunk pass mixes (the chunk
@@ -18,24 +19,35 @@ the groups before it):
 
 Each candidate is timed with the library's kernel events on real parameters;
 the winner is applied to the plan and cached in a JSON file keyed by device
-name and plan shape, so later plans of the same shape skip the search.
-Results do not depend on the tuning (every candidate computes the same sums).
+name, the library whose kernels were timed and plan shape, so later plans of the
+same shape skip the search.  Results do not depend on the tuning (every candidate computes the same sums).
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import os
 
+from .qaoa import LIB_PATH
+
 _DEFAULT_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_tuning_cache.json")
 _FIELDS = ("points_per_task", "blocks_per_sm", "big_scratch_bytes", "reg_bits_grad", "chunk_window")
+
+
+@functools.lru_cache(maxsize=1)
+def _kernels():
+    """Digest of the library: a choice made for other kernels does not answer for these."""
+    with open(LIB_PATH, "rb") as f:
+        return hashlib.sha256(f.read()).hexdigest()[:16]
 
 
 def _key(plan, n_points, grad):
     import torch
     info = plan.info()
     dev = torch.cuda.get_device_name()
-    return (f"{dev}|p={info['p']}|reps={info['n_reps']}|maxq={info['max_qubits']}|maxin={info['max_inner']}"
-            f"|big={info['n_big']}|P={n_points}|grad={int(bool(grad))}")
+    return (f"{dev}|lib={_kernels()}|p={info['p']}|reps={info['n_reps']}|maxq={info['max_qubits']}|maxin={info['max_inner']}"
+            f"|maxe={info['max_edges']}|maxw={plan.max_weight}|big={info['n_big']}|P={n_points}|grad={int(bool(grad))}")
 
 
 def _time(plan, params, grad, reps):
@@ -56,11 +68,9 @@ def candidate_groups(plan, n_points, grad):
     """The groups of tuning values the search walks through, in order: a list
     of lists of partial tunings (dicts over qaoa_tuning_t's fields)."""
     info = plan.info()
-    row_bytes = info["p"] * (info["max_edges"] + 1) * 8
-    jpts = [j for j in (1, 2, 4, 8, 12, 16, 32) if j <= max(1, n_points) and j * row_bytes * 4 <= 48 * 1024]
+    jpts = [j for j in (0, 1, 2, 4, 8, 12, 16, 32) if j <= max(1, n_points)]
     groups = [[{"points_per_task": j, "blocks_per_sm": b} for j in jpts for b in (0, 1, 2)]]
-    # the adjoint register tile matters only to the general register kernel
-    # (depth-1 plans run their register cones on the depth-1 kernel)
+    # depth-1 plans run their register cones on the depth-1 kernel, which has no tile to choose
     has_reg = info["n_reps"] > info["n_big"] and not info["depth1_kernel"]
     if grad and has_reg:
         groups.append([{"reg_bits_grad": r} for r in (4, 5)])

@@ -54,7 +54,7 @@ struct qaoa_device_plan {
     int64_t n_big = 0;
     int32_t points_per_task = 0;  // 0: default (see qaoa_tuning_t)
     int32_t blocks_per_sm = 0;
-    int32_t reg_bits_grad = 0;    // adjoint register qubits (4 or 5; 0: 4)
+    int32_t reg_bits_grad = 0;    // adjoint register qubits (4 or 5; 0: by the amount of work, reg_bits_for)
     int32_t chunk_window = 10;    // largest outer window of a shared-memory chunk pass (6..10)
     bool timing = false;
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> events;

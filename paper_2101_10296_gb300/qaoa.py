@@ -203,6 +203,7 @@ class Plan:
         self.p = p
         self.n_graphs = len(graphs)
         self.n_edges = [int(r.shape[0]) for r in rows]
+        self.max_weight = 1 if weights is None or w.size == 0 else int(np.abs(w).max())
         self._n_reps = None  # filled on first use: a plan's representatives never change
 
     def close(self):
