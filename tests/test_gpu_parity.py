@@ -628,6 +628,41 @@ def test_shared_memory_chunk_windows_match_oracle(q):
     assert plan.device_status() == 0
 
 
+def _alternating_k88():
+    """K_{8,8} with its sides at even and odd vertices, so that a window of outer qubits holds both."""
+    n, e = I.complete_bipartite(8, 8)
+    return n, np.sort(np.where(e < 8, 2 * e, 2 * (e - 8) + 1), axis=1)
+
+
+@pytest.mark.parametrize("graph", [_alternating_k88(), I.wheel(15)], ids=["K88-64-bits", "wheel-30-bits"])
+def test_signed_weights_through_the_chunk_passes(q, graph):
+    """Random signs on K_{8,8} (64 cut bits) and on a wheel of 16 vertices (30) at p = 2: cones of 16 inner
+    qubits, whose windows of six (energy) and seven (adjoint) outer qubits have edges of both signs with
+    both ends inside.  Terms, energies and gradients against the FP64 oracle."""
+    n, edges = graph
+    w = np.random.default_rng(29).choice([1, -1], len(edges))
+    theta = I.draw_params(2, 2, 37)
+    plan = q.Plan(graph, 2, weights=w, orbits=False)
+    reps = plan.reps()
+    big = np.flatnonzero(reps["n_inner"] == 16)
+    assert len(big) >= 15 and all(list(reps["mix_qubits"][r]) == [16, 2] for r in big)
+    _, _, cone_edges = plan.cone(int(big[0]))
+    inside = [int(s) for (a, b), s in zip(cone_edges, plan.cone_weights(int(big[0]))) if min(a, b) >= 10]
+    assert 1 in inside and -1 in inside
+    e, t = plan.energy(_params(theta), terms=True)
+    eg, g, tg = plan.energy_grad(_params(theta), terms=True)
+    adj = O.adjacency(n, edges)
+    for j in range(2):
+        eref, gref = O.orbit_grad_adjoint(n, edges, theta[j], 2, np.arange(len(edges)), adj, weights=w)
+        for x in (e, eg):
+            assert abs(x[0, j].item() - eref) <= E_REL_TOL * len(edges)
+        _check_grad(g[0, j].cpu().numpy(), gref, energy=len(edges))
+        for r in big[:4]:
+            ref = O.lightcone_term(n, edges, edges[reps["edge"][r]], theta[j], 2, adj, weights=w)
+            assert abs(t[r, j].item() - ref) <= TERM_TOL and abs(tg[r, j].item() - ref) <= TERM_TOL
+    assert plan.device_status() == 0
+
+
 def test_chunk_passes_in_many_waves_and_cuda_graph(q):
     """K_{8,8} at p = 2 with 16 points: the chunk passes split into waves of
     two items (1 MiB of scratch) give the results of one wave, and a captured
@@ -1127,6 +1162,39 @@ def test_depth2_kernel_edges(q, graph, weight, P):
             _check_grad(g.cpu().numpy()[0, j], gref, energy=np.abs(w).sum())
     norms = plan.norms(_params(th)).cpu().numpy()
     assert np.abs(norms - 1).max() <= 1e-5
+    assert plan.device_status() == 0
+
+
+@pytest.mark.parametrize("P", [1, 33])
+@pytest.mark.parametrize("graph,weights", [
+    ((2, np.array([[0, 1]])), [31]), ((2, np.array([[0, 1]])), [32]), ((2, np.array([[0, 1]])), [64]),
+    (I.star(8), [1] * 8), (I.star(8), [4] * 7 + [3]), (I.star(8), [4] * 8), (I.star(8), [8] * 8), (I.star(8), [8, -8] * 4)],
+    ids=["edge-31", "edge-32", "edge-64", "star8", "star8-31", "star8-32", "star8-64", "star8-signed-64"])
+def test_depth2_kernel_limits(q, graph, weights, P):
+    """The largest cones the depth-2 kernel takes (nine inner qubits: five on the lanes with four register
+    qubits) and its table rows' last entries (31 cut bits in the narrow rows, 32 and 64 in the wide):
+    terms, energies and both adjoint widths against the FP64 oracle, and every state's norm."""
+    n, edges = graph
+    w = np.array(weights)
+    th = I.draw_params(2, P, 19)
+    plan = q.Plan(graph, 2, weights=[w], orbits=False)
+    info = plan.info()
+    assert info["max_inner"] == n and info["n_big"] == 0
+    e, terms = plan.energy(_params(th), terms=True)
+    scale = np.abs(w).sum()
+    grads = []
+    for bits in (4, 5):
+        plan.set_tuning(reg_bits_grad=bits)
+        grads.append(plan.energy_grad(_params(th)))
+    for j in {0, P - 1}:
+        ref = [O.lightcone_term(n, edges, ed, th[j], 2, weights=w) for ed in edges]
+        assert np.abs(terms.cpu().numpy()[:, j] - ref).max() <= TERM_TOL
+        eref, gref = O.orbit_grad_adjoint(n, edges, th[j], 2, np.arange(len(edges)), weights=w)
+        assert abs(e[0, j].item() - eref) <= E_REL_TOL * scale
+        for eg, g in grads:
+            assert abs(eg[0, j].item() - eref) <= E_REL_TOL * scale
+            _check_grad(g[0, j].cpu().numpy(), gref, energy=scale)
+    assert np.abs(plan.norms(_params(th)).cpu().numpy() - 1).max() <= 1e-5
     assert plan.device_status() == 0
 
 
