@@ -144,7 +144,7 @@ def algorithmic_flops(reps, p, grad, depth1=False):
     elif grad:
         flops = flops + A * (2 + 12 * (ksum - k[:, 0]) + 8 * k[:, 0] + 5 * p + 12 * (p - 1))
         if p <= 3:
-            # the general register kernel (inner parts of <= 9 qubits) takes the last
+            # the register kernels (inner parts of <= 9 qubits) take the last
             # layer's pair terms once when it mixes qubits 0 and 1 only: 2 per
             # amplitude per qubit instead of 4
             last2 = (reps["n_inner"] <= 9) & (k[:, p - 1] == 2)

@@ -392,14 +392,19 @@ int qaoa_device_status(const qaoa_plan *plan, int32_t *status);
  * Launch tuning of a plan (applies to every later call).  Any field 0 means
  * "default".
  *   points_per_task  parameter points one warp task of the register kernels
- *                    evaluates for the same cone slots (default: up to 32,
- *                    while their phase tables fit 8 KB of shared memory;
- *                    larger values are cut to what fits 12 KB per warp; the
- *                    depth-1 kernel's default is what leaves room for its
- *                    resident blocks: the multiprocessor's shared memory
- *                    split among them, less the per-block reservation; the
- *                    depth-2 kernel's gives the busiest multiprocessor the
- *                    least work)
+ *                    evaluates for the same cone slots.  Defaults, all up
+ *                    to 32.  General kernel: while their phase tables fit 8
+ *                    KB of shared memory per warp.  Depth-1 and depth-2
+ *                    kernels: at most what leaves room for their resident
+ *                    blocks (the multiprocessor's shared memory split among
+ *                    them, less the per-block reservation); of these values
+ *                    the depth-2 kernel takes the one that gives the busiest
+ *                    multiprocessor the least work, the others halve theirs
+ *                    while the tasks would not give every multiprocessor 16
+ *                    warps.  Larger values than fit are cut: to 12 KB of
+ *                    tables per warp in the general kernel, to 96 KB per
+ *                    block of four warps in the others, less the reduction
+ *                    buffers and (depth 1) the staged records
  *   blocks_per_sm    resident blocks per SM of the persistent grid (default:
  *                    the occupancy limit)
  *   big_scratch_bytes scratch per call for large-state cones, which sets how

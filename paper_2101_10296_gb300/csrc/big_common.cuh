@@ -129,13 +129,6 @@ __device__ __forceinline__ uint64_t warp_xor(uint64_t x) {
 // c - c0 of a cut value, given b0 = 2^22 + c0 (halves are exact at that size)
 __device__ __forceinline__ float cut_minus(int c, float b0) { return __uint_as_float(0x4A800000u + 2u * uint32_t(c)) - b0; }
 
-__device__ __forceinline__ float lds1(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(v) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ void opaque(uint32_t &v) { asm volatile("" : "+r"(v)); }
-
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return uint32_t(__cvta_generic_to_shared(p)); }
 
 // Rows of a warp's phase tables: 68 real parts, then 68 imaginary parts (a cone
@@ -179,13 +172,6 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
     return v;
-}
-
-// Warp sum in FP32, then one FP64 atomic into base[idx] (energies and terms,
-// whose sums do not cancel).
-__device__ __forceinline__ void add_gp(float v, double *base, int64_t idx) {
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) atomicAdd(base + idx, double(v));
 }
 
 // Compensated warp sum of a derivative partial times w, then one FP64

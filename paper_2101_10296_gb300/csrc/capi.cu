@@ -365,8 +365,6 @@ int build_p1_work(const std::vector<DevCone> &hc, const std::vector<uint64_t> &s
     return QAOA_OK;
 }
 
-RegWork as_reg(const qaoa_device_plan *d, const DevWork &w) { return reg_work(d, w); }
-
 int check_device(const qaoa_plan *plan) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
@@ -413,10 +411,15 @@ namespace qaoa {
 // blocks of four warps); a task costs its points plus about 0.7 of one for its
 // prologue, a multiprocessor with fewer than about `lat` warps waits for
 // latencies as if it had that many, and one in a last, partial round runs no
-// faster than with `min_part`.  Measured against splitting until every
-// multiprocessor had 16 warps and leaving the last task short: random cubic n =
-// 1000, every edge, three points, energy 22.7 -> 18.5 us; n = 1000, 48 points,
-// gradient 393 -> 351 us; n = 200 82 -> 76 us.
+// faster than with `min_part`.  The constants are fitted, to sweeps over all
+// points per task (the two sets of lat and min_part are those of four and of two
+// resident blocks).  The choice against the best of 18 values, on eight plans of
+// 60 to 10,000 vertices (random cubic, signed, 4-regular, a torus) at 3, 10, 25, 48
+// and 100 points, energy and gradient: 0.2% slower in the median, 9% at the ninth
+// decile, 15% at most.  Against splitting until every multiprocessor had 16 warps
+// and leaving the last task short: random cubic n = 1000, every edge, three points,
+// energy 22.7 -> 18.5 us; n = 1000, 48 points, gradient 393 -> 351 us; n = 200 82 ->
+// 76 us.
 int depth2_points(int64_t warps, int64_t n_points, int64_t fit, int blocks_per_sm) {
     const int64_t sms = sm_count();
     const int64_t lat = blocks_per_sm > 2 ? 7 : 4, min_part = blocks_per_sm > 2 ? 10 : 6;
@@ -615,7 +618,7 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
         L.grad = grad;
         L.terms = nullptr;
         L.status = d->status;
-        L.work = as_reg(d, d->reg_p1);
+        L.work = reg_work(d, d->reg_p1);
         // points per warp task: as many phase tables as leave room for
         // kP1PointBlocks resident blocks (a tuned value is held to the kernel's
         // shared-memory limit), halved while the tasks would not give every SM
@@ -658,7 +661,7 @@ int run(const qaoa_plan *plan, int64_t n_points, const double *params, double *e
         L.norm = norm && !grad ? 1 : 0;
         const bool g = grad != nullptr;
         const int rg = g ? reg_bits_for(d, n_points) : kRegBitsEnergy;
-        L.work = as_reg(d, d->reg[rg - 4]);
+        L.work = reg_work(d, d->reg[rg - 4]);
         if (L.work.warps > 0) e = launch_reg(d, L, g, rg, d->points_per_task, s);
         if (L.work.warps > 0) dm->all_launches += 1;
         if (e == cudaSuccess && !d->big.empty()) e = run_big(d, plan, n_points, lut, mix, kpow, energy, grad, terms, norm, cs, fa, s);

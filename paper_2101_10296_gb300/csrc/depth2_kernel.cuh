@@ -64,12 +64,6 @@ __device__ __forceinline__ void mix_q(C2 (&x)[1 << (R - 1)], int q, float tau) {
     }
 }
 
-__device__ __forceinline__ float lds1(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(v) : "r"(addr));
-    return v;
-}
-
 // Counts as bytes.  NARROW (at most 31 cut bits): 4 c, the entry's offset in a
 // 256-byte row (32 real, 32 imaginary parts); otherwise 2 c (c <= 64), rows of
 // kWideRow bytes.
@@ -96,10 +90,6 @@ struct Counts {
         return add2(v, splat(-b0));
     }
 };
-
-// Keeps what is derived from v from being carried in registers from one use to
-// the next (recomputing it is one instruction).
-__device__ __forceinline__ void opaque(uint32_t &v) { asm volatile("" : "+r"(v)); }
 
 template <int R, bool GRAD, bool NARROW>
 __global__ void __launch_bounds__(kRegBlock, depth2_blocks(GRAD, R)) depth2_kernel(const RegLaunch L) {
@@ -221,23 +211,6 @@ __global__ void __launch_bounds__(kRegBlock, depth2_blocks(GRAD, R)) depth2_kern
                     ph[a] = CT::entry(ca, cb, a, row2);
                     y[a] = cmul(x[4 * k + a], ph[a]);
                 }
-                auto mix01 = [](C2(&v)[4], float t) {
-                    C2 a = v[0], b = v[1];
-                    v[0] = bfly(a, b, t);
-                    v[1] = bfly(b, a, t);
-                    a = v[2];
-                    b = v[3];
-                    v[2] = bfly(a, b, t);
-                    v[3] = bfly(b, a, t);
-                    a = v[0];
-                    b = v[2];
-                    v[0] = bfly(a, b, t);
-                    v[2] = bfly(b, a, t);
-                    a = v[1];
-                    b = v[3];
-                    v[1] = bfly(a, b, t);
-                    v[3] = bfly(b, a, t);
-                };
                 mix01(y, tau2);
                 // |y_0|^2 + |y_3|^2 - |y_1|^2 - |y_2|^2 (norm: plus)
                 const P2 pos =

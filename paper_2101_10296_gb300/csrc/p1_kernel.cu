@@ -62,31 +62,6 @@ int occupancy_grid(const void *fn, int block, size_t smem);
 
 namespace {
 
-// (I - i tau X) on qubit 0 (pairs (0,1), (2,3)), then on qubit 1 ((0,2), (1,3))
-__device__ __forceinline__ void mix01(C2 (&x)[4], float tau) {
-    C2 a = x[0], b = x[1];
-    x[0] = bfly(a, b, tau);
-    x[1] = bfly(b, a, tau);
-    a = x[2];
-    b = x[3];
-    x[2] = bfly(a, b, tau);
-    x[3] = bfly(b, a, tau);
-    a = x[0];
-    b = x[2];
-    x[0] = bfly(a, b, tau);
-    x[2] = bfly(b, a, tau);
-    a = x[1];
-    b = x[3];
-    x[1] = bfly(a, b, tau);
-    x[3] = bfly(b, a, tau);
-}
-
-__device__ __forceinline__ float lds1(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(v) : "r"(addr));
-    return v;
-}
-
 // Table row layouts: SMALL up to 32 entries (256 bytes: real parts, imaginary
 // parts from byte 128), MID up to 64 (512 bytes, from byte 256), both with the
 // count bytes scaled by 4 and the row at a multiple of 256, so that the byte

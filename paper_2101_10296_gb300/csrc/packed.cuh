@@ -82,10 +82,38 @@ __device__ __forceinline__ C2 swap(const C2 &a) { return C2{swap(a.r), swap(a.i)
 __device__ __forceinline__ C2 bfly(const C2 &u, const C2 &v, float tau) {
     return C2{fma2(splat(tau), v.i, u.r), fma2(splat(-tau), v.r, u.i)};
 }
+// (I - i tau X) on qubit 0 (pairs (0,1), (2,3)), then on qubit 1 ((0,2), (1,3))
+__device__ __forceinline__ void mix01(C2 (&x)[4], float tau) {
+    C2 a = x[0], b = x[1];
+    x[0] = bfly(a, b, tau);
+    x[1] = bfly(b, a, tau);
+    a = x[2];
+    b = x[3];
+    x[2] = bfly(a, b, tau);
+    x[3] = bfly(b, a, tau);
+    a = x[0];
+    b = x[2];
+    x[0] = bfly(a, b, tau);
+    x[2] = bfly(b, a, tau);
+    a = x[1];
+    b = x[3];
+    x[1] = bfly(a, b, tau);
+    x[3] = bfly(b, a, tau);
+}
 __device__ __forceinline__ P2 shfl_xor(P2 a, int m) {
     const float2 h = halves(a);
     return p2(__shfl_xor_sync(0xffffffffu, h.x, m), __shfl_xor_sync(0xffffffffu, h.y, m));
 }
 __device__ __forceinline__ C2 shfl_xor(const C2 &a, int m) { return C2{shfl_xor(a.r, m), shfl_xor(a.i, m)}; }
+
+// Four bytes at a shared-memory address.
+__device__ __forceinline__ float lds1(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(v) : "r"(addr));
+    return v;
+}
+// Keeps what is derived from v from being carried in registers from one use to
+// the next (recomputing it is one instruction).
+__device__ __forceinline__ void opaque(uint32_t &v) { asm volatile("" : "+r"(v)); }
 
 }  // namespace qaoa
